@@ -186,7 +186,7 @@ NCU_FP64_FLOPS = {
 def kernel_source_hash():
     """sha256 of the kernel source and the build script (its flags)."""
     h = hashlib.sha256()
-    for rel in (("csrc", "fr_kernels.cuh"), ("build.py",)):
+    for rel in (("csrc", "fr_kernels.cuh"), ("csrc", "fr_line.cuh"), ("build.py",)):
         with open(os.path.join(ROOT, "paper_2312_14167_gb300", *rel), "rb") as f:
             h.update(f.read())
     return h.hexdigest()

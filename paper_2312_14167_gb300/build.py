@@ -48,7 +48,7 @@ def _flags(debug=False):
 def _stale(obj, src):
     if not os.path.exists(obj):
         return True
-    deps = [src, os.path.join(CSRC, "fr_kernels.cuh"), os.path.join(CSRC, "fr_internal.h"),
+    deps = [src, os.path.join(CSRC, "fr_kernels.cuh"), os.path.join(CSRC, "fr_line.cuh"), os.path.join(CSRC, "fr_internal.h"),
             os.path.join(ROOT, "include", "fr.h")]
     t = os.path.getmtime(obj)
     return any(os.path.getmtime(d) > t for d in deps if os.path.exists(d))

@@ -92,6 +92,7 @@ struct Group {
     // fused viscous stage: second (ping-pong) buffer of the inbound gradient
     // flux parts (the first is FV) and the partner lifting coefficients
     char *FV2 = nullptr, *LFP = nullptr;
+    char *FGEO = nullptr;   // FP32 fused stage: packed face geometry
     // adaptive steps: third RK register (u_n) and the group's first element
     // in the batch's per-element error array
     char *R3 = nullptr;
@@ -296,7 +297,7 @@ Plan make_plan(fr_mesh *const *meshes, int n_inst) {
 }
 
 struct GroupLayout {
-    size_t U, R1, R2, RES, UF0, UF1, FV, MET, NRM, MFLUX, PART, EINST, WALL, DIVREF, FV2, LFP, R3;
+    size_t U, R1, R2, RES, UF0, UF1, FV, MET, NRM, MFLUX, PART, EINST, WALL, DIVREF, FV2, LFP, R3, FGEO;
 };
 struct Layout {
     GroupLayout g[frk::kMaxGroups];
@@ -333,6 +334,7 @@ Layout make_layout(const Plan &P, int n_inst, bool fp64, bool visc, bool adapt) 
         G.FV2 = take(visc ? fc : 16);
         G.LFP = take(visc ? (size_t)E * nfp * dim * rs : 16);
         G.R3 = take(adapt ? st : 16);
+        G.FGEO = take(visc && !fp64 && dim == 2 ? (size_t)E * nfp * frk::kFaceGeo * 4 : 16);
     }
     L.BTAG = take((size_t)P.nb * 4);
     L.BVREF = take((size_t)P.nb * dim * rs);
@@ -403,6 +405,8 @@ void fill_args(const fr_solver *s, int g, frk::KArgs<real> &a) {
     a.DIVREF = G.use_divref ? (const real *)G.DIVREF : nullptr;
     a.FLAGS = s->FLAGS;
     a.LFP = (const real *)G.LFP;
+    a.FGEO = (const float *)G.FGEO;
+    a.kq = (real)((s->visc ? s->cfg.mu : 0.0) * s->cfg.gamma / (s->cfg.prandtl > 0 ? s->cfg.prandtl : 1.0));
     a.local_ref = s->local_ref ? 1 : 0;
     a.regs_level = s->regs_level;
     a.tc = (s->tc && !s->fp64) ? 1 : 0;
@@ -425,8 +429,27 @@ void fill_args(const fr_solver *s, int g, frk::KArgs<real> &a) {
         a.opGL[i] = r.dgL[i];
         a.opGR[i] = r.dgR[i];
         a.opW[i] = r.w[i];
+        a.rL[i] = (real)r.lend[0][i];
+        a.rL[frk::kMaxN + i] = (real)r.lend[1][i];
+        a.rGL[i] = (real)r.dgL[i];
+        a.rGR[i] = (real)r.dgR[i];
+        for (int mm = 0; mm < G.N; ++mm) {
+            a.rD[i * frk::kMaxN + mm] = (real)r.D1[i][mm];
+            a.rDT[i * frk::kMaxN + mm] =
+                (real)(r.D1[i][mm] - r.dgR[i] * r.lend[1][mm] - r.dgL[i] * r.lend[0][mm]);
+        }
         for (int mm = 0; mm < G.N; ++mm)
             a.opDT[i * frk::kMaxN + mm] = r.D1[i][mm] - r.dgR[i] * r.lend[1][mm] - r.dgL[i] * r.lend[0][mm];
+    }
+    auto pair = [](real c) { return make_float2((float)c, (float)c); };
+    for (int i = 0; i < frk::kMaxN * frk::kMaxN; ++i) {
+        a.rD2[i] = pair(a.rD[i]);
+        a.rDT2[i] = pair(a.rDT[i]);
+    }
+    for (int i = 0; i < 2 * frk::kMaxN; ++i) a.rL2[i] = pair(a.rL[i]);
+    for (int i = 0; i < frk::kMaxN; ++i) {
+        a.rGLm2[i] = pair(-a.rGL[i]);
+        a.rGR2[i] = pair(a.rGR[i]);
     }
 }
 
@@ -991,7 +1014,8 @@ template <typename real>
 void to_real(std::vector<char> &dst, const std::vector<double> &src) {
     dst.resize(src.size() * sizeof(real));
     real *d = reinterpret_cast<real *>(dst.data());
-    for (size_t i = 0; i < src.size(); ++i) d[i] = (real)src[i];
+#pragma omp parallel for schedule(static) if (src.size() > 100000)
+    for (int64_t i = 0; i < (int64_t)src.size(); ++i) d[i] = (real)src[i];
 }
 }  // namespace
 
@@ -1059,6 +1083,7 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
         G.FV2 = w + gl.FV2;
         G.LFP = w + gl.LFP;
         G.R3 = w + gl.R3;
+        G.FGEO = w + gl.FGEO;
     }
     s->BTAG = (int32_t *)(w + L.BTAG); s->BVREF = w + L.BVREF;
     s->stage64 = (double *)(w + L.STAGE);
@@ -1275,10 +1300,15 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
         }
         FR_CK(cudaMemsetAsync(G.MFLUX, 0, (size_t)G.n_box * s->V * s->rsz, cs));
     }
-    // BR2 stages may run as one fused kernel when every face is conforming;
-    // the default is the gradient + flux kernel pair, fr_tune measures both
+    // BR2 stages may run as one fused kernel when every face is conforming.
+    // That is the default where it is the line kernel (2-D FP32, p >= 1:
+    // measured faster than the gradient + flux pair at every size, 2.50 against
+    // 4.89 ms per step on 32 airfoil-sized O-meshes of p = 3, 0.142 against
+    // 0.236 ms on 31,722 quads); elsewhere and for adaptive steps the pair is,
+    // and fr_tune measures both
     const bool fusable = s->visc && cfg->viscous_scheme == FR_VISC_BR2 && P.n_mortar == 0;
-    s->fused = false;
+    s->fused = fusable && !s->fp64 && !s->adapt && dim == 2;
+    for (int g = 0; g < P.G; ++g) s->fused = s->fused && s->grp[g].N >= 2;
     if (fusable) {
         // partner lifting coefficients per own flux point (FP64, then cast):
         // lf = sum_m l_m(side) g'_side(m) (1/J) S[k][:] along the partner's line
@@ -1298,12 +1328,32 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
                         for (int jd = 0; jd < dim; ++jd) lf[((size_t)e * nfp + f) * dim + jd] += c * Mv[k * dim + jd];
                     }
                 }
-            for (size_t q = 0; q < (size_t)G.E * nfp; ++q) {
+#pragma omp parallel for schedule(static)
+            for (int64_t q = 0; q < G.E * nfp; ++q) {
                 const int32_t pt = part[g][q];
                 if (pt < 0) continue;
                 for (int jd = 0; jd < dim; ++jd) lfp[q * dim + jd] = lf[(size_t)pt * dim + jd];
             }
             FR_CK(up_real(G.LFP, lfp, lfp.size()));
+            if (!s->fp64 && dim == 2) {
+                // the line kernel's face record: normal, own and partner lifting
+                // coefficients times eta, partner index
+                const double eta = cfg->br2_eta > 0 ? cfg->br2_eta : 2.0 * dim;
+                std::vector<float> rec((size_t)G.E * nfp * frk::kFaceGeo, 0.0f);
+#pragma omp parallel for schedule(static)
+                for (int64_t q = 0; q < G.E * nfp; ++q) {
+                    // [face][part][point], two parts of four values
+                    const int64_t face = q / G.nfpf, l = q % G.nfpf;
+                    float *A = &rec[(size_t)((2 * face) * G.nfpf + l) * 4], *B = A + 4 * G.nfpf;
+                    for (int d = 0; d < 2; ++d) {
+                        A[d] = (float)nrm[g][(size_t)q * 2 + d];
+                        A[2 + d] = (float)(eta * lf[(size_t)q * 2 + d]);
+                        B[d] = (float)(eta * lfp[(size_t)q * 2 + d]);
+                    }
+                    std::memcpy(B + 2, &part[g][q], 4);
+                }
+                FR_CK(up(G.FGEO, rec.data(), rec.size() * 4));
+            }
         }
     }
     if (!s->fp64) {

@@ -28,6 +28,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <climits>
+#include <type_traits>
 
 namespace frk {
 
@@ -66,6 +67,7 @@ enum Mode : int {
     M_BS_START = 8,    // fresh instances: R1 = R, R3 = u
     M_BS_2 = 9,        // R2 = R; u = R3 + (3/4) h R
     M_BS_3 = 10,       // u = R3 + h (2/9 R1 + 1/3 R2 + 4/9 R); RES = -5/72 R1 + 1/12 R2 + 1/9 R
+    M_FACES = 12,      // no evaluation: face data of the current state (K_INTERP_VISC of the line kernel)
     M_BS_4 = 11,       // R2 = R (state unchanged); K_BS_ERROR then sums the error h (RES - R2/8)
 };
 
@@ -175,6 +177,11 @@ struct KArgs {
     // in: DT[i][m] = D1[i][m] - g_R'(xi_i) l_m(+1) - g_L'(xi_i) l_m(-1)
     double opDT[kMaxN * kMaxN];
     double opW[kMaxN];            // Gauss weights
+    // the same in the kernel's precision, read from the constant bank (K_LINE)
+    real rD[kMaxN * kMaxN], rDT[kMaxN * kMaxN], rL[2 * kMaxN], rGL[kMaxN], rGR[kMaxN];
+    float2 rD2[kMaxN * kMaxN], rDT2[kMaxN * kMaxN], rL2[2 * kMaxN], rGLm2[kMaxN], rGR2[kMaxN];   // as pairs (c, c); -g_L'
+    real kq;                      // gamma mu / Pr
+    const float *FGEO;            // packed face geometry of K_LINE [E][face][2][point][4]
     // perturbation storage (FP32 kernels): reference state, its FP64
     // conserved values (for the FP64 staging conversions and integrals), and
     // J times the residual of the constant reference flux per solution point
@@ -2295,6 +2302,10 @@ k_interp_visc(const KArgs<real> a) {
     send_faces<D, N, PAD>(a, sU, sG, Lm, Lp, e0, ne);
 }
 
+}  // namespace frk
+#include "fr_line.cuh"
+namespace frk {
+
 // --------------------------------------------------------------------------
 // K_INTERP: face values of the current state (after fr_set_state)
 // --------------------------------------------------------------------------
@@ -2955,10 +2966,15 @@ template <int D, int N, typename real>
 cudaError_t launch_n(int kind, bool visc, const KArgs<real> &a, int grid_hint, cudaStream_t st) {
     using G = Geo<D, N>;
     const int64_t tiles = (a.n_elem + G::NE - 1) / G::NE;
+    const bool ad = a.ADAPT != nullptr;   // adaptive steps: their own instantiation, register level 0
     const bool l1 = has_level1<N, real>() && a.regs_level == 1;
     const bool l2 = has_level1<N, real>() && a.regs_level == 2;
     constexpr int R1 = has_level1<N, real>() ? 1 : 0, R2 = has_level1<N, real>() ? 2 : 0;
-    const bool ad = a.ADAPT != nullptr;   // adaptive steps: their own instantiation, register level 0
+    // 2-D FP32 fused stages run the line kernel; the tensor-core option and
+    // adaptive steps keep K_STAGE (an adaptive run on the stability limit
+    // amplifies a change of rounding to 5e-5 of the state within 40 attempts,
+    // so its kernels stay as they are, bit for bit)
+    const bool line_stage = has_line<D, N, real>() && !a.tc && !ad;
     if (kind == K_FLUX) {
         if (a.n_elem <= 0) return cudaSuccess;
         const size_t sm = smem_bytes<D, N, real>(K_FLUX, visc, a.tc != 0);
@@ -2992,6 +3008,17 @@ cudaError_t launch_n(int kind, bool visc, const KArgs<real> &a, int grid_hint, c
         cudaError_t err = prep_smem(k, sm);
         if (err != cudaSuccess) return err;
         k<<<(unsigned)tiles, G::THREADS, sm, st>>>(a);
+    } else if (line_stage && (kind == K_STAGE || kind == K_INTERP_VISC)) {
+        if (a.n_elem <= 0) return cudaSuccess;
+        if constexpr (has_line<D, N, real>()) {
+            KArgs<real> b = a;
+            if (kind == K_INTERP_VISC) b.mode = M_FACES;
+            using L = Line2<N>;
+            auto k = l2 ? k_line2<N, R2> : l1 ? k_line2<N, R1> : k_line2<N, 0>;
+            cudaError_t err = prep_smem(k, L::BYTES);
+            if (err != cudaSuccess) return err;
+            k<<<(unsigned)((a.n_elem + L::EPB - 1) / L::EPB), L::TH, L::BYTES, st>>>(b);
+        }
     } else if (kind == K_STAGE) {
         if (a.n_elem <= 0) return cudaSuccess;
         const size_t sm = smem_bytes<D, N, real>(K_STAGE, true, a.tc != 0);

@@ -1,0 +1,61 @@
+"""The line kernel of 2-D FP32 BR2 stages (one thread per element row and
+column, a warp per 32 // (p + 1) elements) against the FP64 oracle at the
+edges of its tiles: element counts around one warp and one CTA, every degree,
+neighbouring faces in every orientation, both interface fluxes.
+
+Residuals: the standard forward error bound of the FP32 sums on the path's own
+FP32 input (16 roundings of the terms' magnitude).  Steps: 1e-6 of the state,
+the bound of the mixed path's short horizons."""
+import numpy as np
+import pytest
+
+from tests import fr_cases as FC
+from oracle import timestep as T
+from synth import meshes as M
+
+pytestmark = pytest.mark.gpu
+
+EPS32 = 2.0 ** -24
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+def _case(shape, p, flux="rusanov", rk="lsrk45"):
+    mesh = M.reorient(M.periodic_box(2, shape, (0.0, 0.0), (1.0, 0.9), jitter=0.2), 5)
+    return FC.Case("line", [mesh], p, True, 0.01, 0.3, dt=1e-4, flux=flux, rk=rk)
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+@pytest.mark.parametrize("shape", [(3, 3), (8, 4), (11, 3), (5, 13)])
+def test_residual_at_tile_edges(shape, p):
+    case = _case(shape, p, flux="roe" if shape[0] == 8 else "rusanov")
+    sol = FC.lib_solver(case, "fp32")
+    assert "stage=fused" in sol.schedule()[0]
+    disc = FC.oracle_disc(case)
+    u = FC.initial_state(case, disc.sol_coords())
+    sol.set_state(0, u)
+    R32, mag = disc.residual(FC.fp32_input(case, u), magnitude=True)
+    err = FC.rel_l2(sol.residual(0), R32)
+    bound = 16 * EPS32 * np.linalg.norm(mag) / np.linalg.norm(R32)
+    print(f"p={p} {shape}: {err:.2e} (bound {bound:.2e})")
+    assert err < bound
+
+
+@pytest.mark.parametrize("rk", ["rk4", "lsrk45"])
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+def test_steps_follow_the_oracle(p, rk):
+    case = _case((11, 3), p, rk=rk)
+    sol = FC.lib_solver(case, "fp32")
+    disc = FC.oracle_disc(case)
+    u = FC.initial_state(case, disc.sol_coords())
+    sol.set_state(0, u)
+    sol.rk_step(5)
+    step = T.rk4_step if rk == "rk4" else T.lsrk45_step
+    for _ in range(5):
+        u = step(disc.residual, u, case.dt)
+    assert FC.rel_l2(sol.get_state(0), u) < 1e-6
