@@ -92,7 +92,7 @@ struct Group {
     // fused viscous stage: second (ping-pong) buffer of the inbound gradient
     // flux parts (the first is FV) and the partner lifting coefficients
     char *FV2 = nullptr, *LFP = nullptr;
-    char *FGEO = nullptr;   // FP32 fused stage: packed face geometry
+    char *FGEO = nullptr, *METL = nullptr;   // FP32 fused stage: packed face geometry, reordered metric terms (3-D)
     // adaptive steps: third RK register (u_n) and the group's first element
     // in the batch's per-element error array
     char *R3 = nullptr;
@@ -297,7 +297,7 @@ Plan make_plan(fr_mesh *const *meshes, int n_inst) {
 }
 
 struct GroupLayout {
-    size_t U, R1, R2, RES, UF0, UF1, FV, MET, NRM, MFLUX, PART, EINST, WALL, DIVREF, FV2, LFP, R3, FGEO;
+    size_t U, R1, R2, RES, UF0, UF1, FV, MET, NRM, MFLUX, PART, EINST, WALL, DIVREF, FV2, LFP, R3, FGEO, METL;
 };
 struct Layout {
     GroupLayout g[frk::kMaxGroups];
@@ -334,7 +334,8 @@ Layout make_layout(const Plan &P, int n_inst, bool fp64, bool visc, bool adapt) 
         G.FV2 = take(visc ? fc : 16);
         G.LFP = take(visc ? (size_t)E * nfp * dim * rs : 16);
         G.R3 = take(adapt ? st : 16);
-        G.FGEO = take(visc && !fp64 && dim == 2 ? (size_t)E * nfp * frk::kFaceGeo * 4 : 16);
+        G.FGEO = take(visc && !fp64 ? (size_t)E * nfp * frk::face_geo(dim) * 4 : 16);
+        G.METL = take(visc && !fp64 && dim == 3 ? (size_t)E * nsp * MS * 4 : 16);
     }
     L.BTAG = take((size_t)P.nb * 4);
     L.BVREF = take((size_t)P.nb * dim * rs);
@@ -406,6 +407,7 @@ void fill_args(const fr_solver *s, int g, frk::KArgs<real> &a) {
     a.FLAGS = s->FLAGS;
     a.LFP = (const real *)G.LFP;
     a.FGEO = (const float *)G.FGEO;
+    a.METL = (const float *)G.METL;
     a.kq = (real)((s->visc ? s->cfg.mu : 0.0) * s->cfg.gamma / (s->cfg.prandtl > 0 ? s->cfg.prandtl : 1.0));
     a.local_ref = s->local_ref ? 1 : 0;
     a.regs_level = s->regs_level;
@@ -1084,6 +1086,7 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
         G.LFP = w + gl.LFP;
         G.R3 = w + gl.R3;
         G.FGEO = w + gl.FGEO;
+        G.METL = w + gl.METL;
     }
     s->BTAG = (int32_t *)(w + L.BTAG); s->BVREF = w + L.BVREF;
     s->stage64 = (double *)(w + L.STAGE);
@@ -1301,13 +1304,14 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
         FR_CK(cudaMemsetAsync(G.MFLUX, 0, (size_t)G.n_box * s->V * s->rsz, cs));
     }
     // BR2 stages may run as one fused kernel when every face is conforming.
-    // That is the default where it is the line kernel (2-D FP32, p >= 1:
-    // measured faster than the gradient + flux pair at every size, 2.50 against
-    // 4.89 ms per step on 32 airfoil-sized O-meshes of p = 3, 0.142 against
-    // 0.236 ms on 31,722 quads); elsewhere and for adaptive steps the pair is,
-    // and fr_tune measures both
+    // That is the default where it is a line kernel (FP32, p >= 1: measured
+    // faster than the gradient + flux pair at every size, ms per step 2.50
+    // against 4.89 on 32 airfoil-sized O-meshes of p = 3, 0.142 against 0.236
+    // on 31,722 quads, 3.3 against 5.9 on 48^3 hexes of p = 3, 4.7 against 6.8
+    // on 57,120 of p = 4); elsewhere and for adaptive steps the pair is, and
+    // fr_tune measures both
     const bool fusable = s->visc && cfg->viscous_scheme == FR_VISC_BR2 && P.n_mortar == 0;
-    s->fused = fusable && !s->fp64 && !s->adapt && dim == 2;
+    s->fused = fusable && !s->fp64 && !s->adapt;
     for (int g = 0; g < P.G; ++g) s->fused = s->fused && s->grp[g].N >= 2;
     if (fusable) {
         // partner lifting coefficients per own flux point (FP64, then cast):
@@ -1335,24 +1339,34 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
                 for (int jd = 0; jd < dim; ++jd) lfp[q * dim + jd] = lf[(size_t)pt * dim + jd];
             }
             FR_CK(up_real(G.LFP, lfp, lfp.size()));
-            if (!s->fp64 && dim == 2) {
+            if (!s->fp64) {
                 // the line kernel's face record: normal, own and partner lifting
                 // coefficients times eta, partner index
                 const double eta = cfg->br2_eta > 0 ? cfg->br2_eta : 2.0 * dim;
-                std::vector<float> rec((size_t)G.E * nfp * frk::kFaceGeo, 0.0f);
+                std::vector<float> rec((size_t)G.E * nfp * frk::face_geo(dim), 0.0f);
 #pragma omp parallel for schedule(static)
                 for (int64_t q = 0; q < G.E * nfp; ++q) {
-                    // [face][part][point], two parts of four values
+                    // [face][part][point], dim parts of four values
                     const int64_t face = q / G.nfpf, l = q % G.nfpf;
-                    float *A = &rec[(size_t)((2 * face) * G.nfpf + l) * 4], *B = A + 4 * G.nfpf;
-                    for (int d = 0; d < 2; ++d) {
-                        A[d] = (float)nrm[g][(size_t)q * 2 + d];
-                        A[2 + d] = (float)(eta * lf[(size_t)q * 2 + d]);
-                        B[d] = (float)(eta * lfp[(size_t)q * 2 + d]);
+                    float *A = &rec[(size_t)((dim * face) * G.nfpf + l) * 4], *B = A + 4 * G.nfpf, *C = B + 4 * G.nfpf;
+                    for (int d = 0; d < dim; ++d) {
+                        A[d] = (float)nrm[g][(size_t)q * dim + d];
+                        (dim == 2 ? A + 2 : B)[d] = (float)(eta * lf[(size_t)q * dim + d]);
+                        (dim == 2 ? B : C)[d] = (float)(eta * lfp[(size_t)q * dim + d]);
                     }
-                    std::memcpy(B + 2, &part[g][q], 4);
+                    std::memcpy(dim == 2 ? B + 2 : A + 3, &part[g][q], 4);
                 }
                 FR_CK(up(G.FGEO, rec.data(), rec.size() * 4));
+                if (dim == 3) {
+                    std::vector<float> ml((size_t)G.E * nsp * MS);
+#pragma omp parallel for schedule(static)
+                    for (int64_t e = 0; e < G.E; ++e)
+                        for (int sp = 0; sp < nsp; ++sp)
+                            for (int c = 0; c < MS; ++c)
+                                ml[(size_t)frk::metl_word(N, G.E, e, sp % N, c, sp / N)] =
+                                    (float)met[g][((size_t)e * nsp + sp) * MS + c];
+                    FR_CK(up(G.METL, ml.data(), ml.size() * 4));
+                }
             }
         }
     }
@@ -2517,8 +2531,10 @@ extern "C" fr_status fr_tune(fr_solver *s, const char *cache_path, int mode, cha
         return st;
     }
     const Cand *best = &cands[0];
+    // at the resolution reported below: of candidates that run alike (register
+    // levels of a kernel that has one, or of a batch smaller than the chip) the first
     for (const Cand &c : cands)
-        if (c.ms < best->ms) best = &c;
+        if (std::llround(c.ms * 1e4) < std::llround(best->ms * 1e4)) best = &c;
     char v[160];
     std::snprintf(v, sizeof(v), "stage=%s;regs=%d;contract=%s;ms=%.6f", best->fused ? "fused" : "split", best->regs,
                   best->tc ? "tc" : "simt", best->ms);

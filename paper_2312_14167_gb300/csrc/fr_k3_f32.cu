@@ -33,6 +33,8 @@ static cudaError_t prepare_n(bool visc) {
     e = prep_smem(k_stage<3, N, float, 0, true>, smem_bytes<3, N, float>(K_STAGE, true));
     if (e != cudaSuccess) return e;
     e = prep_smem(k_interp_visc<3, N, float>, smem_bytes<3, N, float>(K_INTERP_VISC, true));
+    if constexpr (has_line<3, N, float>())
+        if (e == cudaSuccess) e = prep_smem(k_line3<N>, Line3<N>::BYTES);
     if (e != cudaSuccess || !has_level1<N, float>()) return e;
     // register level 1 (autotuner candidates)
     constexpr int L1 = has_level1<N, float>() ? 1 : 0;

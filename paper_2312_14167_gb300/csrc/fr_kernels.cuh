@@ -181,7 +181,8 @@ struct KArgs {
     real rD[kMaxN * kMaxN], rDT[kMaxN * kMaxN], rL[2 * kMaxN], rGL[kMaxN], rGR[kMaxN];
     float2 rD2[kMaxN * kMaxN], rDT2[kMaxN * kMaxN], rL2[2 * kMaxN], rGLm2[kMaxN], rGR2[kMaxN];   // as pairs (c, c); -g_L'
     real kq;                      // gamma mu / Pr
-    const float *FGEO;            // packed face geometry of K_LINE [E][face][2][point][4]
+    const float *FGEO;            // packed face geometry of K_LINE [E][face][D][point][4]
+    const float *METL;            // K_LINE, 3-D: metric terms, order of metl_word
     // perturbation storage (FP32 kernels): reference state, its FP64
     // conserved values (for the FP64 staging conversions and integrals), and
     // J times the residual of the constant reference flux per solution point
@@ -2970,7 +2971,7 @@ cudaError_t launch_n(int kind, bool visc, const KArgs<real> &a, int grid_hint, c
     const bool l1 = has_level1<N, real>() && a.regs_level == 1;
     const bool l2 = has_level1<N, real>() && a.regs_level == 2;
     constexpr int R1 = has_level1<N, real>() ? 1 : 0, R2 = has_level1<N, real>() ? 2 : 0;
-    // 2-D FP32 fused stages run the line kernel; the tensor-core option and
+    // FP32 fused stages run the line kernels; the tensor-core option and
     // adaptive steps keep K_STAGE (an adaptive run on the stability limit
     // amplifies a change of rounding to 5e-5 of the state within 40 attempts,
     // so its kernels stay as they are, bit for bit)
@@ -3013,8 +3014,10 @@ cudaError_t launch_n(int kind, bool visc, const KArgs<real> &a, int grid_hint, c
         if constexpr (has_line<D, N, real>()) {
             KArgs<real> b = a;
             if (kind == K_INTERP_VISC) b.mode = M_FACES;
-            using L = Line2<N>;
-            auto k = l2 ? k_line2<N, R2> : l1 ? k_line2<N, R1> : k_line2<N, 0>;
+            using L = std::conditional_t<D == 2, Line2<N>, Line3<N>>;
+            void (*k)(const KArgs<float>);
+            if constexpr (D == 2) k = l2 ? k_line2<N, R2> : l1 ? k_line2<N, R1> : k_line2<N, 0>;
+            else k = k_line3<N>;   // one register level: two CTAs per SM by shared memory
             cudaError_t err = prep_smem(k, L::BYTES);
             if (err != cudaSuccess) return err;
             k<<<(unsigned)((a.n_elem + L::EPB - 1) / L::EPB), L::TH, L::BYTES, st>>>(b);

@@ -1,17 +1,17 @@
-// K_LINE: the fused BR2 Navier-Stokes stage of 2-D FP32 solvers, one thread
-// per element line (included by fr_kernels.cuh).
+// K_LINE: the fused BR2 Navier-Stokes stage of FP32 solvers, one thread per
+// element line (included by fr_kernels.cuh).
 //
 // Same method and exchange as K_STAGE (every element sends its partners its
 // face state and the gradient part of its viscous normal flux; the next stage
 // forms both sides' BR2 fluxes locally), with another split of the work.  A
-// thread owns one row and one column of its element, so everything
+// thread owns one line of every direction of its element, so everything
 // one-dimensional - derivative, interpolation to the line's two faces,
 // divergence with its correction - runs on registers with operator entries
 // from the constant bank, and a value goes through shared memory once per
-// direction instead of N times.  The threads of an element sit in one warp:
-// no CTA barrier separates the phases.
+// direction instead of N times.  The threads of an element sit in one warp
+// (25-line hexes: one CTA): no CTA barrier separates the phases.
 //
-// Measured (GB300, p = 3, 259,298 curved quads, one stage): gradient + flux
+// 2-D, measured (GB300, p = 3, 259,298 curved quads, one stage): gradient + flux
 // kernels 306 us (1,500 instructions per point, issue slots and phase barriers
 // the bound); one thread per line 193 us (777 instructions; the L1 data stage,
 // 36 % of its cycles on 64-byte-step row accesses); rows and face data fetched
@@ -23,10 +23,11 @@
 
 namespace frk {
 
-// values per flux point of the packed face geometry: outward normal (scaled
-// by |dS|) and own lifting coefficients (times eta); partner's lifting
-// coefficients, partner index as bits, unused
-constexpr int kFaceGeo = 8;
+// values per flux point of the packed face geometry, in parts of four: 2-D
+// normal (outward, scaled by |dS|) and own lifting coefficients (times eta),
+// then the partner's and its index as bits; 3-D normal and partner index, own
+// lifting coefficients, the partner's
+__host__ __device__ constexpr int face_geo(int dim) { return 4 * dim; }
 
 // NV contiguous values of a row at a multiple of NV values (so 16-byte aligned
 // where NV is a multiple of 4, 8-byte aligned where it is even)
@@ -418,6 +419,13 @@ __device__ __forceinline__ void cp16(void *dst, const void *src) {
 __device__ __forceinline__ void cp4(void *dst, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
                  : "memory");
+}
+__device__ __forceinline__ void cp8(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void prefetch_l2(const void *src) {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(src));
 }
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int K>
@@ -866,8 +874,488 @@ k_line2(const __grid_constant__ KArgs<float> a) {
     send(1);
 }
 
+// --------------------------------------------------------------------------
+// 3-D line kernel.  A thread owns line l of each of the three directions of
+// its element.  A state or flux of five variables is one 128-bit vector (rho,
+// rho v) and one word (rho E), in shared memory as in the face buffers.
+// Loops over directions and points stay rolled where their bodies are long:
+// unrolled, the kernel is 7,200 instructions that every warp runs once, and
+// instruction fetch was the largest stall (p = 4: 4 of 10 cycles per issue).
+// Metric terms come in an order of their own, so that neighbouring lanes read
+// neighbouring vectors; they, the partners' states and viscous fluxes are
+// fetched at the start by asynchronous copies, the face geometry and the RK
+// register prefetched into L2.  Shared memory then holds two CTAs per SM,
+// which leaves 255 registers a thread (three CTAs at 168 spill 260 bytes and
+// measured 8 % slower).
+//
+// Measured (GB300, ms per LSRK45 step), gradient + flux kernels at their best
+// register level -> this kernel: 48^3 hexes of p = 3 5.32 -> 3.12, 57,120 of
+// p = 4 6.62 -> 4.59.  On the way (p = 3): unrolled, one plane per variable
+// 4.56; loops rolled 3.90; vectors 3.43; staged inputs 3.29; prefetches 3.12.
+// Bound by latency at 8 warps per SM: 44 % of the issue slots, 55 % of the L1
+// data stage, 35 % of DRAM at p = 3.
+// --------------------------------------------------------------------------
+template <int N>
+struct Line3 {
+    static constexpr int V = 5, MS = 10, NSP = N * N * N, LPE = N * N, NFP = 6 * LPE;
+    static constexpr int TH = 128;
+    static constexpr bool WARP = LPE <= 16;             // an element's lines fit a warp
+    static constexpr int EPW = WARP ? 32 / LPE : 1;
+    static constexpr int EPB = WARP ? EPW * (TH / 32) : TH / LPE;
+    // slot of point (i, j, k): i + SJ j + SK k, SE per element.  N = 4: with a
+    // row of 5 slots every 128-bit phase of a row or column view and every
+    // 32-bit access of them falls in different banks (the zeta view: one
+    // conflict in eight lanes)
+    static constexpr int SJ = N == 4 ? 5 : N, SK = N * SJ, SE = N * SK;
+    static constexpr int NS = EPB * SE;                 // slots of a field
+    static constexpr int ND = EPB * LPE;                // face jumps of one (direction, side)
+    // fields: 0 state, 1..3 gradient / transformed flux; then the jumps of
+    // directions 1, 2.  Vectors first, the fifth variable behind them
+    static constexpr int SLOTS = 4 * NS + 4 * ND;
+    // staged inputs: metric terms (two vectors and a pair per point), then the
+    // partners' states and viscous fluxes (a vector and a word per flux point)
+    static constexpr int NF = EPB * NFP, NM = EPB * NSP;
+    static constexpr int oM = SLOTS, oUF = oM + 2 * NM, oFV = oUF + NF, VECS = oFV + NF;      // vectors
+    static constexpr int oMC = (SLOTS + 1) / 2 * 2, oUE = oMC + 2 * NM, oFE = oUE + NF, TAILS = oFE + NF;   // words
+    static constexpr size_t BYTES = (size_t)VECS * 16 + (size_t)TAILS * 4;
+    static_assert(BYTES <= 115712, "two CTAs per SM");
+    __device__ __forceinline__ static int step(int k) { return k == 0 ? 1 : (k == 1 ? SJ : SK); }
+    __device__ __forceinline__ static int base(int k, int l) {
+        return k == 0 ? (l % N) * SJ + (l / N) * SK : l % N + (l / N) * (k == 1 ? SK : SJ);
+    }
+};
+// word of metric term c at point i of xi line `line` of element e of n_elem:
+// [element][point of the line][two vectors of all lines], then [element][point]
+// [one pair of all lines]
+__host__ __device__ constexpr int64_t metl_word(int N, int64_t n_elem, int64_t e, int i, int c, int line) {
+    return c < 8 ? (((e * N + i) * 2 + c / 4) * (N * N) + line) * 4 + c % 4
+                 : n_elem * N * N * N * 8 + ((e * N + i) * (N * N) + line) * 2 + c - 8;
+}
+
+// Five variables, four of them as packed pairs (see V4)
+struct V5 {
+    V4 p;
+    float c;
+    __device__ __forceinline__ void get(float *x) const {
+        p.get(x);
+        x[4] = c;
+    }
+};
+__device__ __forceinline__ V5 fma5(const float2 k, const float *x, const V5 &t) {
+    return V5{fma4(k, x, t.p), fmaf(k.x, x[4], t.c)};
+}
+__device__ __forceinline__ V5 mul5(const float2 k, const float *x) { return V5{mul4(k, x), k.x * x[4]}; }
+
+// face data of the 3-D line kernel: the vectors of all nf flux points, then
+// their fifth variables
+__device__ __forceinline__ void st_face3(float *buf, int64_t nf, int32_t pt, const float *o) {
+    reinterpret_cast<float4 *>(buf)[pt] = make_float4(o[0], o[1], o[2], o[3]);
+    buf[4 * nf + pt] = o[4];
+}
+
+template <int N>
+__global__ void __launch_bounds__((Line3<N>::TH), 2)
+k_line3(const __grid_constant__ KArgs<float> a) {
+    using L = Line3<N>;
+    using real = float;
+    constexpr int D = 3, V = 5, NSP = L::NSP, LPE = L::LPE, MS = L::MS, NS = L::NS;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float4 *sv = reinterpret_cast<float4 *>(smem_raw);
+    real *se = reinterpret_cast<real *>(sv + L::VECS);
+    const int tid = threadIdx.x;
+    const int64_t e_end = a.elem0 + a.n_elem, eb = a.elem0 + (int64_t)blockIdx.x * L::EPB;
+    const int ne = (int)min((int64_t)L::EPB, e_end - eb);
+    // element slot and line of this thread; threads without an element of
+    // their own repeat another one's line and store nothing
+    int j, l;
+    bool live;
+    if (L::WARP) {
+        const int w = (tid >> 5) * L::EPW, x = (tid & 31) / LPE;
+        if (w >= ne) return;                       // whole warps: only warp barriers below
+        l = (tid & 31) % LPE;
+        live = x < L::EPW && w + x < ne;
+        j = live ? w + x : w;
+    } else {
+        j = tid / LPE;
+        l = tid % LPE;
+        live = j < ne;
+        j = live ? j : 0;
+    }
+    auto sync = [] {
+        if (L::WARP) __syncwarp();
+        else __syncthreads();
+    };
+    const int64_t e = eb + j;
+    const int la = l % N, lb = l / N;
+    const int mode = a.mode;
+    const real gm1 = a.gamma - real(1), kq = a.kq;
+    const int64_t nf = a.fp_real;                  // flux points of the group
+    {
+        // the group's inputs (a warp's or the CTA's elements g0 .. g0 + gn)
+        const int t0 = L::WARP ? tid & 31 : tid, nt = L::WARP ? 32 : L::TH;
+        const int g0 = L::WARP ? (tid >> 5) * L::EPW : 0, gn = min(L::WARP ? L::EPW : L::EPB, ne - g0);
+        const float4 *mA = reinterpret_cast<const float4 *>(a.METL) + (eb + g0) * (2 * NSP);
+        const float2 *mC = reinterpret_cast<const float2 *>(a.METL + nf / L::NFP * NSP * 8) + (eb + g0) * NSP;
+        for (int i = t0; i < gn * 2 * NSP; i += nt) cp16(sv + L::oM + g0 * 2 * NSP + i, mA + i);
+        for (int i = t0; i < gn * NSP; i += nt) cp8(se + L::oMC + 2 * (g0 * NSP + i), mC + i);
+        cp_commit();
+        if (mode != M_FACES) {
+            const int64_t f0 = (eb + g0) * L::NFP;
+            for (int i = t0; i < gn * L::NFP; i += nt) {
+                cp16(sv + L::oUF + g0 * L::NFP + i, a.UFin + 4 * (f0 + i));
+                cp16(sv + L::oFV + g0 * L::NFP + i, a.FVin + 4 * (f0 + i));
+                cp4(se + L::oUE + g0 * L::NFP + i, a.UFin + 4 * nf + f0 + i);
+                cp4(se + L::oFE + g0 * L::NFP + i, a.FVin + 4 * nf + f0 + i);
+            }
+        }
+        cp_commit();
+        // what is read later from memory: into L2 meanwhile (128-byte lines)
+        const char *pg = reinterpret_cast<const char *>(a.FGEO) + (eb + g0) * (L::NFP * 48);
+        for (int i = t0 * 128; i < gn * L::NFP * 48; i += nt * 128) prefetch_l2(pg + i);
+        if (mode == M_LSRK) {
+            const char *pr = reinterpret_cast<const char *>(a.R1 + (eb + g0) * (NSP * V));
+            for (int i = t0 * 128; i < gn * NSP * V * 4; i += nt * 128) prefetch_l2(pr + i);
+        }
+    }
+    const float4 *mA = sv + L::oM + j * 2 * NSP + l;
+    const float2 *mC = reinterpret_cast<const float2 *>(se + L::oMC) + j * NSP + l;
+    auto met = [&](int i, real *M) {
+        const float4 A = mA[2 * i * LPE], B = mA[(2 * i + 1) * LPE];
+        const float2 C = mC[i * LPE];
+        M[0] = A.x; M[1] = A.y; M[2] = A.z; M[3] = A.w; M[4] = B.x; M[5] = B.y; M[6] = B.z; M[7] = B.w;
+        M[8] = C.x; M[9] = C.y;
+    };
+    auto ld = [&](int slot, real *o) {
+        const float4 t = sv[slot];
+        o[0] = t.x; o[1] = t.y; o[2] = t.z; o[3] = t.w;
+        o[4] = se[slot];
+    };
+    auto st = [&](int slot, const real *o) {
+        if (!live) return;
+        sv[slot] = make_float4(o[0], o[1], o[2], o[3]);
+        se[slot] = o[4];
+    };
+    auto deriv = [&](int i, const real (*x)[V], real *o) {
+        V5 t = mul5(a.rD2[i * kMaxN], x[0]);
+#pragma unroll
+        for (int m = 1; m < N; ++m) t = fma5(a.rD2[i * kMaxN + m], x[m], t);
+        t.get(o);
+    };
+    auto ends = [&](const real (*x)[V], real (*o)[V]) {
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            V5 t = mul5(a.rL2[s * kMaxN], x[0]);
+#pragma unroll
+            for (int m = 1; m < N; ++m) t = fma5(a.rL2[s * kMaxN + m], x[m], t);
+            t.get(o[s]);
+        }
+    };
+    const int ju = j * L::SE, jr = ju + L::base(0, l);     // the element's first slot, the row's
+    const int64_t row = (e * NSP + l * N) * V;
+    real u[N][V];
+    ld_row<N * V>(a.U + row, &u[0][0]);
+#pragma unroll
+    for (int m = 0; m < N; ++m) st(jr + m, u[m]);
+    cp_wait<1>();
+    sync();
+
+#pragma unroll 1
+    for (int pass = mode == M_FACES ? 1 : 0; pass < 2; ++pass) {
+        // uncorrected physical gradient of the state (u, field U) at every point into the fields G
+#pragma unroll 1
+        for (int k = 1; k < D; ++k) {
+            const int o = ju + L::base(k, l), so = L::step(k);
+            real x[N][V];
+#pragma unroll
+            for (int m = 0; m < N; ++m) ld(o + m * so, x[m]);
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                real d[V];
+                deriv(i, x, d);
+                st(k * NS + o + i * so, d);
+            }
+        }
+        sync();
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            real M[MS], dk[D][V];
+            met(i, M);
+            deriv(i, u, dk[0]);
+            ld(NS + jr + i, dk[1]);
+            ld(2 * NS + jr + i, dk[2]);
+#pragma unroll
+            for (int d = 0; d < D; ++d) {
+                real g[V];
+                const real c0 = M[d] * M[9], c1 = M[3 + d] * M[9], c2 = M[6 + d] * M[9];
+#pragma unroll
+                for (int v = 0; v < V; ++v) g[v] = c0 * dk[0][v] + c1 * dk[1][v] + c2 * dk[2][v];
+                st((1 + d) * NS + jr + i, g);
+            }
+        }
+        sync();
+
+        if (pass == 1) {
+            // 4) face state + gradient flux part of the (new) state to the
+            // partners' inbound slots for the next stage
+#pragma unroll 1
+            for (int k = 0; k < D; ++k) {
+                const int o = ju + L::base(k, l), so = L::step(k);
+                const int64_t face = e * 6 + 2 * k;
+                float4 geo[2];
+#pragma unroll
+                for (int s = 0; s < 2; ++s)
+                    geo[s] = __ldg(reinterpret_cast<const float4 *>(a.FGEO) + (face + s) * (3 * LPE) + l);
+                real uf[2][V], Q[2][D][V];
+                {
+                    real x[N][V];
+#pragma unroll
+                    for (int m = 0; m < N; ++m) ld(o + m * so, x[m]);
+                    ends(x, uf);
+                }
+#pragma unroll
+                for (int d = 0; d < D; ++d) {
+                    real x[N][V], q[2][V];
+#pragma unroll
+                    for (int m = 0; m < N; ++m) ld((1 + d) * NS + o + m * so, x[m]);
+                    ends(x, q);
+#pragma unroll
+                    for (int s = 0; s < 2; ++s)
+#pragma unroll
+                        for (int v = 0; v < V; ++v) Q[s][d][v] = q[s][v];
+                }
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    const int32_t pt = __float_as_int(geo[s].w);
+                    if (!live || pt < 0) continue;
+                    const real n[D] = {geo[s].x, geo[s].y, geo[s].z};
+                    real full[V], v[D], fv[V];
+                    add_ref<V>(a.ref, uf[s], full);
+                    const real ir = real(1) / full[0];
+#pragma unroll
+                    for (int d = 0; d < D; ++d) v[d] = full[1 + d] * ir;
+                    visc_normal<D>(Q[s], v, full[V - 1] * ir, a.mu * ir, kq * ir, n, fv);
+                    st_face3(a.UFout, nf, pt, uf[s]);
+                    st_face3(a.FVout, nf, pt, fv);
+                }
+            }
+            return;
+        }
+
+        LineRef<D, real> R;      // the element's flux reference, its own or the global one
+        {
+            real u0[V];
+            ld(ju, u0);
+            line_ref<D>(a.ref, u0, a.local_ref && !a.DIVREF, a.gamma, R);
+        }
+        // 1) common normal fluxes and jumps at the ends of this thread's lines
+        cp_wait<0>();
+        sync();
+        real F0[2][V], F1[2][V], F2[2][V], dd0[2][V];
+#pragma unroll 1
+        for (int k = 0; k < D; ++k) {
+            const int64_t face = e * 6 + 2 * k;
+            FaceGeo<D, real> g[2];
+            real uR[2][V], fvp[2][V];
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                const float4 *p = reinterpret_cast<const float4 *>(a.FGEO) + (face + s) * (3 * LPE) + l;
+                const float4 A = __ldg(p), B = __ldg(p + LPE), C = __ldg(p + 2 * LPE);
+                g[s].n[0] = A.x; g[s].n[1] = A.y; g[s].n[2] = A.z; g[s].pt = __float_as_int(A.w);
+                g[s].lf[0] = B.x; g[s].lf[1] = B.y; g[s].lf[2] = B.z;
+                g[s].lfp[0] = C.x; g[s].lfp[1] = C.y; g[s].lfp[2] = C.z;
+                const int q = j * L::NFP + (2 * k + s) * LPE + l;
+                const float4 U = sv[L::oUF + q], W = sv[L::oFV + q];
+                uR[s][0] = U.x; uR[s][1] = U.y; uR[s][2] = U.z; uR[s][3] = U.w; uR[s][4] = se[L::oUE + q];
+                fvp[s][0] = W.x; fvp[s][1] = W.y; fvp[s][2] = W.z; fvp[s][3] = W.w; fvp[s][4] = se[L::oFE + q];
+            }
+            const int o = ju + L::base(k, l), so = L::step(k);
+            real uf[2][V], Q[2][D][V];
+            {
+                real x[N][V];
+#pragma unroll
+                for (int m = 0; m < N; ++m) ld(o + m * so, x[m]);
+                ends(x, uf);
+            }
+#pragma unroll
+            for (int d = 0; d < D; ++d) {
+                real x[N][V], q[2][V];
+#pragma unroll
+                for (int m = 0; m < N; ++m) ld((1 + d) * NS + o + m * so, x[m]);
+                ends(x, q);
+#pragma unroll
+                for (int s = 0; s < 2; ++s)
+#pragma unroll
+                    for (int v = 0; v < V; ++v) Q[s][d][v] = q[s][v];
+            }
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                real F[V], dd[V];
+                line_face<D, N>(a, R, g[s], uf[s], Q[s], uR[s], fvp[s], kq, F, dd);
+                if (k == 0) {
+#pragma unroll
+                    for (int v = 0; v < V; ++v) { F0[s][v] = F[v]; dd0[s][v] = dd[v]; }
+                } else {
+                    st(4 * NS + ((k - 1) * 2 + s) * L::ND + j * LPE + l, dd);
+#pragma unroll
+                    for (int v = 0; v < V; ++v) {
+                        if (k == 1) F1[s][v] = F[v];
+                        else F2[s][v] = F[v];
+                    }
+                }
+            }
+        }
+        sync();
+
+        // 2) transformed flux at the points of the xi line, corrected gradient
+        {
+            const real g1l = a.rGL[la], g1r = a.rGR[la], g2l = a.rGL[lb], g2r = a.rGR[lb];
+            const int jd = 4 * NS + j * LPE;
+#pragma unroll 1
+            for (int i = 0; i < N; ++i) {
+                real M[MS], ui[V], gr[D][V], d1m[V], d1p[V], d2m[V], d2p[V];
+                met(i, M);
+                ld(jr + i, ui);
+#pragma unroll
+                for (int d = 0; d < D; ++d) ld((1 + d) * NS + jr + i, gr[d]);
+                ld(jd + i + N * lb, d1m);
+                ld(jd + L::ND + i + N * lb, d1p);
+                ld(jd + 2 * L::ND + i + N * la, d2m);
+                ld(jd + 3 * L::ND + i + N * la, d2p);
+                const real g0l = a.rGL[i], g0r = a.rGR[i];
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    const real c0 = M[9] * (g0l * dd0[0][v] + g0r * dd0[1][v]);
+                    const real c1 = M[9] * (g1l * d1m[v] + g1r * d1p[v]);
+                    const real c2 = M[9] * (g2l * d2m[v] + g2r * d2p[v]);
+#pragma unroll
+                    for (int d = 0; d < D; ++d) gr[d][v] += M[d] * c0 + M[3 + d] * c1 + M[6 + d] * c2;
+                }
+                real F[D][V];
+                line_flux<D>(a, R, ui, gr, gm1, kq, F);
+#pragma unroll
+                for (int k = 0; k < D; ++k) {
+                    real t[V];
+#pragma unroll
+                    for (int v = 0; v < V; ++v) t[v] = M[3 * k] * F[0][v] + M[3 * k + 1] * F[1][v] + M[3 * k + 2] * F[2][v];
+                    st((1 + k) * NS + jr + i, t);
+                }
+            }
+        }
+        sync();
+
+        // 3) divergence + correction along every line (the flux polynomial's
+        // end values are folded into DT), then the RK update of the xi line
+        auto div_pt = [&](int i, const real (*x)[V], const real (*F)[V], real *o) {
+            V5 t = fma5(a.rGLm2[i], F[0], mul5(a.rGR2[i], F[1]));
+#pragma unroll
+            for (int m = 0; m < N; ++m) t = fma5(a.rDT2[i * kMaxN + m], x[m], t);
+            t.get(o);
+        };
+        real r1[N][V];           // issued here: its latency passes under the divergence
+        if (mode == M_LSRK) ld_row<N * V>(a.R1 + row, &r1[0][0]);
+#pragma unroll 1
+        for (int k = 1; k < D; ++k) {
+            const int o = (1 + k) * NS + ju + L::base(k, l), so = L::step(k);
+            real x[N][V], F[2][V];
+#pragma unroll
+            for (int m = 0; m < N; ++m) ld(o + m * so, x[m]);
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+#pragma unroll
+                for (int v = 0; v < V; ++v) F[s][v] = k == 1 ? F1[s][v] : F2[s][v];
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                real d[V];
+                div_pt(i, x, F, d);
+                st(o + i * so, d);
+            }
+        }
+        real dv[N][V];
+        {
+            real x[N][V];
+#pragma unroll
+            for (int m = 0; m < N; ++m) ld(NS + jr + m, x[m]);
+#pragma unroll
+            for (int i = 0; i < N; ++i) div_pt(i, x, F0, dv[i]);
+        }
+        sync();
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            real x[V], y[V];
+            ld(2 * NS + jr + i, x);
+            ld(3 * NS + jr + i, y);
+#pragma unroll
+            for (int v = 0; v < V; ++v) dv[i][v] += x[v] + y[v];
+        }
+        if (a.DIVREF) {
+            // the constant reference flux's share of the divergence
+            real dr[N][V];
+            ld_row<N * V>(a.DIVREF + row, &dr[0][0]);
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+#pragma unroll
+                for (int v = 0; v < V; ++v) dv[i][v] += dr[i][v];
+        }
+        if (mode == M_RESIDUAL_J) {
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+#pragma unroll
+                for (int v = 0; v < V; ++v) dv[i][v] = -dv[i][v];
+            if (live) st_row<N * V>(a.RES + row, &dv[0][0]);
+            return;
+        }
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const real iJ = mC[i * LPE].y;
+#pragma unroll
+            for (int v = 0; v < V; ++v) dv[i][v] *= -iJ;
+        }
+        if (mode == M_RESIDUAL) {
+            if (live) st_row<N * V>(a.RES + row, &dv[0][0]);
+            return;
+        }
+        if (mode == M_LSRK_FIRST || mode == M_LSRK) {
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    r1[i][v] = mode == M_LSRK ? a.rk_a * r1[i][v] + a.dt * dv[i][v] : a.dt * dv[i][v];
+                    u[i][v] += a.rk_b * r1[i][v];
+                }
+            if (live) st_row<N * V>(a.R1 + row, &r1[0][0]);
+        } else if (mode == M_RK4_1) {
+            if (live) {
+                st_row<N * V>(a.R1 + row, &u[0][0]);
+                st_row<N * V>(a.R2 + row, &dv[0][0]);
+            }
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+#pragma unroll
+                for (int v = 0; v < V; ++v) u[i][v] += a.rk_c * dv[i][v];
+        } else {
+            real r2[N][V];
+            ld_row<N * V>(a.R1 + row, &r1[0][0]);
+            ld_row<N * V>(a.R2 + row, &r2[0][0]);
+            const bool last = mode == M_RK4_4;
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    const real acc = last ? r2[i][v] + dv[i][v] : r2[i][v] + real(2) * dv[i][v];
+                    u[i][v] = r1[i][v] + a.rk_c * (last ? acc : dv[i][v]);
+                    r2[i][v] = acc;
+                }
+            if (live && !last) st_row<N * V>(a.R2 + row, &r2[0][0]);
+        }
+        if (live) st_row<N * V>(a.U + row, &u[0][0]);
+#pragma unroll
+        for (int i = 0; i < N; ++i) st(jr + i, u[i]);
+        sync();
+    }
+}
+
 // does this launch use the line kernel?
 template <int D, int N, typename real>
-__host__ __device__ constexpr bool has_line() { return D == 2 && sizeof(real) == 4 && N >= 2; }
+__host__ __device__ constexpr bool has_line() { return sizeof(real) == 4 && N >= 2; }
 
 }  // namespace frk

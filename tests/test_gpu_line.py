@@ -1,7 +1,7 @@
-"""The line kernel of 2-D FP32 BR2 stages (one thread per element row and
-column, a warp per 32 // (p + 1) elements) against the FP64 oracle at the
-edges of its tiles: element counts around one warp and one CTA, every degree,
-neighbouring faces in every orientation, both interface fluxes.
+"""The line kernels of FP32 BR2 stages (one thread per element line of every
+direction) against the FP64 oracle at the edges of their tiles: element counts
+around one warp and one CTA, every degree, neighbouring faces in every
+orientation, both interface fluxes.
 
 Residuals: the standard forward error bound of the FP32 sums on the path's own
 FP32 input (16 roundings of the terms' magnitude).  Steps: 1e-6 of the state,
@@ -26,14 +26,15 @@ def _cuda():
 
 
 def _case(shape, p, flux="rusanov", rk="lsrk45"):
-    mesh = M.reorient(M.periodic_box(2, shape, (0.0, 0.0), (1.0, 0.9), jitter=0.2), 5)
-    return FC.Case("line", [mesh], p, True, 0.01, 0.3, dt=1e-4, flux=flux, rk=rk)
+    dim = len(shape)
+    mesh = M.reorient(M.periodic_box(dim, shape, (0.0,) * dim, (1.0, 0.9, 1.1)[:dim], jitter=0.2), 5)
+    return FC.Case("line", [mesh], p, True, 0.01, 0.3, dt=1e-4, flux=flux, rk=rk, v_inf=(1.0, 0.0, 0.0)[:dim])
 
 
 @pytest.mark.parametrize("p", [1, 2, 3, 4])
-@pytest.mark.parametrize("shape", [(3, 3), (8, 4), (11, 3), (5, 13)])
+@pytest.mark.parametrize("shape", [(3, 3), (8, 4), (11, 3), (5, 13), (3, 3, 3), (4, 4, 3), (3, 5, 7)])
 def test_residual_at_tile_edges(shape, p):
-    case = _case(shape, p, flux="roe" if shape[0] == 8 else "rusanov")
+    case = _case(shape, p, flux="roe" if shape[0] in (8, 4) else "rusanov")
     sol = FC.lib_solver(case, "fp32")
     assert "stage=fused" in sol.schedule()[0]
     disc = FC.oracle_disc(case)
@@ -48,9 +49,11 @@ def test_residual_at_tile_edges(shape, p):
 
 @pytest.mark.parametrize("rk", ["rk4", "lsrk45"])
 @pytest.mark.parametrize("p", [1, 2, 3, 4])
-def test_steps_follow_the_oracle(p, rk):
-    case = _case((11, 3), p, rk=rk)
+@pytest.mark.parametrize("shape", [(11, 3), (3, 3, 5)])
+def test_steps_follow_the_oracle(shape, p, rk):
+    case = _case(shape, p, rk=rk)
     sol = FC.lib_solver(case, "fp32")
+    assert "stage=fused" in sol.schedule()[0]
     disc = FC.oracle_disc(case)
     u = FC.initial_state(case, disc.sol_coords())
     sol.set_state(0, u)
