@@ -132,6 +132,7 @@ template <typename real>
 struct KArgs {
     int64_t n_elem;            // elements (or list entries) in the launch
     int64_t elem0;             // first element of the launch range
+    int tile;                  // elements per CTA of the tile kernels, at most Geo::NE (tile_elems)
     const int32_t *elist;      // optional element list (force sampling)
     real *U, *R1, *R2, *RES;
     const real *UFin;          // [E][NFP][V] inbound: the partner's face state at each own point
@@ -324,21 +325,41 @@ __device__ __forceinline__ void flux_normal(const real *u, const real *n, real g
     c2 = gamma * p / rho;
 }
 
+// An FP64 division or square root costs about ten FMA-pipe instructions, so
+// the wave speed is taken as lambda |n| = max |v.n| + sqrt(|n|^2 c^2) with c^2
+// from the reciprocal density that the velocities need anyway: two divisions
+// and two square roots per point instead of six and three.
+template <int D, typename real>
+__device__ __forceinline__ real normal_flux_speed(const real *u, const real *n, real nn, real gamma, real *F) {
+    const real ir = real(1) / u[0];
+    real vel[D], ke = 0, vn = 0;
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+        vel[i] = u[1 + i] * ir;
+        ke += vel[i] * u[1 + i];
+        vn += vel[i] * n[i];
+    }
+    const real p = (gamma - real(1)) * (u[D + 1] - real(0.5) * ke);
+    F[0] = u[0] * vn;
+#pragma unroll
+    for (int i = 0; i < D; ++i) F[1 + i] = u[1 + i] * vn + p * n[i];
+    F[D + 1] = (u[D + 1] + p) * vn;
+    return fabs(vn) + sqrt(nn * (gamma * p * ir));
+}
+
 template <int D, typename real>
 __device__ __forceinline__ void rusanov(const real *uL, const real *uR, const real *n,
                                         real gamma, real *F) {
     constexpr int V = D + 2;
-    const real gm1 = gamma - real(1);
     real nn = 0;
 #pragma unroll
     for (int j = 0; j < D; ++j) nn += n[j] * n[j];
-    const real nm = sqrt(nn);
-    real FL[V], FR[V], vnL, vnR, c2L, c2R;
-    flux_normal<D>(uL, n, gm1, FL, vnL, c2L, gamma);
-    flux_normal<D>(uR, n, gm1, FR, vnR, c2R, gamma);
-    const real lam = fmax(fabs(vnL) / nm + sqrt(c2L), fabs(vnR) / nm + sqrt(c2R));
+    real FL[V], FR[V];
+    const real sL = normal_flux_speed<D>(uL, n, nn, gamma, FL);
+    const real sR = normal_flux_speed<D>(uR, n, nn, gamma, FR);
+    const real lam = real(0.5) * fmax(sL, sR);
 #pragma unroll
-    for (int v = 0; v < V; ++v) F[v] = real(0.5) * (FL[v] + FR[v]) - real(0.5) * (lam * nm) * (uR[v] - uL[v]);
+    for (int v = 0; v < V; ++v) F[v] = real(0.5) * (FL[v] + FR[v]) - lam * (uR[v] - uL[v]);
 }
 
 // Roe's approximate Riemann solver (n scaled by |dS|): Roe-averaged state,
@@ -457,6 +478,87 @@ __device__ __forceinline__ void flux_vis(const real *u, const real (*grad)[D + 2
         for (int k = 0; k < D; ++k) vdv += vel[k] * gv[j][k];
         // -q_j = (mu/Pr) d/dx_j (E + p/rho - v.v/2) = (mu/Pr) gamma (dE/dx_j - v_k dv_k/dx_j)
         F[j][D + 1] = work + kq * (gE[j] - vdv);
+    }
+}
+
+// viscous normal flux of the gradient Q for a state given by 1/rho, v and
+// specific energy Es; mi = mu / rho, ki = gamma mu / Pr / rho
+template <int D, typename real>
+__device__ __forceinline__ void visc_normal(const real (*Q)[D + 2], const real *v, real Es, real mi, real ki,
+                                            const real *n, real *out) {
+    constexpr int V = D + 2;
+    // rho times the velocity gradient [j][i] = d v_i / d x_j and, along n, the
+    // gradients of v and E
+    real gv[D][D], an[D], div = 0, qn0 = 0, qnE = 0;
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+#pragma unroll
+        for (int i = 0; i < D; ++i) gv[j][i] = Q[j][1 + i] - Q[j][0] * v[i];
+        div += gv[j][j];
+        qn0 += n[j] * Q[j][0];
+        qnE += n[j] * Q[j][V - 1];
+    }
+    real work = 0, va = 0;
+    const real d3 = real(2.0 / 3.0) * div;
+    out[0] = 0;
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+        real a = 0, b = 0;
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+            a += n[j] * gv[j][i];
+            b += n[j] * gv[i][j];
+        }
+        an[i] = a;
+        out[1 + i] = mi * (a + b - d3 * n[i]);
+        work += v[i] * out[1 + i];
+        va += v[i] * an[i];
+    }
+    out[V - 1] = work + ki * (qnE - qn0 * Es - va);
+}
+
+// F(u) - F_v(u, grad u) in every direction (FP64): one reciprocal, and the
+// velocity gradients kept times rho
+template <int D, typename real>
+__device__ __forceinline__ void flux_total(const real *u, const real (*gr)[D + 2], real gm1, real mu, real kq,
+                                           real (*F)[D + 2]) {
+    constexpr int V = D + 2;
+    const real ir = real(1) / u[0];
+    real v[D], ke = 0;
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+        v[i] = u[1 + i] * ir;
+        ke += v[i] * u[1 + i];
+    }
+    const real p = gm1 * (u[V - 1] - real(0.5) * ke), H = u[V - 1] + p;
+    const real Es = u[V - 1] * ir, mi = mu * ir, ki = kq * ir;
+    real gv[D][D], div = 0;
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+#pragma unroll
+        for (int c = 0; c < D; ++c) gv[d][c] = gr[d][1 + c] - gr[d][0] * v[c];
+        div += gv[d][d];
+    }
+    const real d3 = real(2.0 / 3.0) * div;
+    real tau[D][D];
+#pragma unroll
+    for (int d = 0; d < D; ++d)
+#pragma unroll
+        for (int c = d; c < D; ++c) {
+            tau[d][c] = mi * (c == d ? gv[d][d] + gv[d][d] - d3 : gv[d][c] + gv[c][d]);
+            tau[c][d] = tau[d][c];
+        }
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+        F[d][0] = u[1 + d];
+        real wk = 0, va = 0;
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+            F[d][1 + c] = u[1 + c] * v[d] + ((c == d ? p : real(0)) - tau[d][c]);
+            wk += v[c] * tau[d][c];
+            va += v[c] * gv[d][c];
+        }
+        F[d][V - 1] = H * v[d] - wk - ki * (gr[d][V - 1] - gr[d][0] * Es - va);
     }
 }
 
@@ -1198,10 +1300,10 @@ k_grad(const KArgs<real> a) {
     real *sGD = sB + pad4(NE * NFP * V);      // [j][s][jd][v], V pad floats per row if PAD
     const real *D1 = sOp, *Lm = sOp + N * N, *Lp = Lm + N, *GL = Lp + N, *GR = GL + N;
 
-    const int64_t e0 = a.elem0 + (int64_t)blockIdx.x * NE;
+    const int64_t e0 = a.elem0 + (int64_t)blockIdx.x * a.tile;
     const int64_t e_end = a.elem0 + a.n_elem;
     if (e0 >= e_end) return;
-    const int ne = (int)min((int64_t)NE, e_end - e0);
+    const int ne = (int)min((int64_t)a.tile, e_end - e0);
     const int tid = threadIdx.x;
 
     // face data of this thread's flux points, issued first: partner index,
@@ -1349,21 +1451,24 @@ k_grad(const KArgs<real> a) {
         for (int jd = 0; jd < D; ++jd)
 #pragma unroll
             for (int v = 0; v < V; ++v) Q[jd][v] += eta * lf[jd] * dd[v];
-        real Fv[D][V];
-        real ubf[V];
-        if constexpr (PERT) add_ref<V>(a.ref, ub, ubf);
-        else {
-#pragma unroll
-            for (int v = 0; v < V; ++v) ubf[v] = ub[v];
-        }
-        flux_vis<D>(ubf, Q, a.gamma, a.mu, a.prandtl, Fv);
         real fvn[V];
+        if constexpr (PERT) {
+            real Fv[D][V], ubf[V];
+            add_ref<V>(a.ref, ub, ubf);
+            flux_vis<D>(ubf, Q, a.gamma, a.mu, a.prandtl, Fv);
 #pragma unroll
-        for (int v = 0; v < V; ++v) {
-            real t = 0;
+            for (int v = 0; v < V; ++v) {
+                real t = 0;
 #pragma unroll
-            for (int d = 0; d < D; ++d) t += Fv[d][v] * nr[it][d];
-            fvn[v] = t;
+                for (int d = 0; d < D; ++d) t += Fv[d][v] * nr[it][d];
+                fvn[v] = t;
+            }
+        } else {
+            const real ir = real(1) / ub[0];
+            real vel[D];
+#pragma unroll
+            for (int d = 0; d < D; ++d) vel[d] = ub[1 + d] * ir;
+            visc_normal<D>(Q, vel, ub[V - 1] * ir, a.mu * ir, a.kq * ir, nr[it], fvn);
         }
         const bool wall = pt[it] < 0 && a.BTAG[-1 - pt[it]] == BC_WALL;
         if (wall) fvn[V - 1] = 0;
@@ -1473,10 +1578,10 @@ k_flux(const KArgs<real> a) {
     real *sDiv = sF + pad4(NE * D * NSP * V) + lr_slots<D, N, real>();   // [k][j][s][v] (tensor-core option)
     const real *D1 = sOp, *Lm = sOp + N * N, *Lp = Lm + N, *GL = Lp + N, *GR = GL + N, *DT = GR + N;
 
-    const int64_t e0 = a.elem0 + (int64_t)blockIdx.x * NE;
+    const int64_t e0 = a.elem0 + (int64_t)blockIdx.x * a.tile;
     const int64_t e_end = a.elem0 + a.n_elem;
     if (e0 >= e_end) return;
-    const int ne = (int)min((int64_t)NE, e_end - e0);
+    const int ne = (int)min((int64_t)a.tile, e_end - e0);
     const int tid = threadIdx.x;
     const int mode = a.mode;
 
@@ -1623,7 +1728,7 @@ k_flux(const KArgs<real> a) {
 #pragma unroll
             for (int v = 0; v < V; ++v) ul[v] = uu[v] - sLR[j].du[v];
             flux_inv_pert<D>(ul, sLR[j].r, a.gamma - real(1), F);
-        } else {
+        } else if (!VISC) {
             flux_inv<D>(uu, a.gamma - real(1), F);
         }
         if (VISC) {
@@ -1658,18 +1763,17 @@ k_flux(const KArgs<real> a) {
                     for (int k = 0; k < D; ++k) g += M[k * D + jd] * Gk[k][v];
                     gr[jd][v] = g * iJ;
                 }
-            real Fv[D][V];
-            real uf[V];
-            if constexpr (PERT) add_ref<V>(a.ref, uu, uf);
-            else {
+            if constexpr (PERT) {
+                real Fv[D][V], uf[V];
+                add_ref<V>(a.ref, uu, uf);
+                flux_vis<D>(uf, gr, a.gamma, a.mu, a.prandtl, Fv);
 #pragma unroll
-                for (int v = 0; v < V; ++v) uf[v] = uu[v];
+                for (int jd = 0; jd < D; ++jd)
+#pragma unroll
+                    for (int v = 0; v < V; ++v) F[jd][v] -= Fv[jd][v];
+            } else {
+                flux_total<D>(uu, gr, a.gamma - real(1), a.mu, a.kq, F);
             }
-            flux_vis<D>(uf, gr, a.gamma, a.mu, a.prandtl, Fv);
-#pragma unroll
-            for (int jd = 0; jd < D; ++jd)
-#pragma unroll
-                for (int v = 0; v < V; ++v) F[jd][v] -= Fv[jd][v];
         }
 #pragma unroll
         for (int k = 0; k < D; ++k) {
@@ -1946,10 +2050,10 @@ k_stage(const KArgs<real> a) {
     real *sDiv = sF + pad4(NE * D * NSP * V) + lr_slots<D, N, real>();   // [k][j][s][v] (tensor-core option)
     const real *D1 = sOp, *Lm = sOp + N * N, *Lp = Lm + N, *GL = Lp + N, *GR = GL + N, *DT = GR + N;
 
-    const int64_t e0 = a.elem0 + (int64_t)blockIdx.x * NE;
+    const int64_t e0 = a.elem0 + (int64_t)blockIdx.x * a.tile;
     const int64_t e_end = a.elem0 + a.n_elem;
     if (e0 >= e_end) return;
-    const int ne = (int)min((int64_t)NE, e_end - e0);
+    const int ne = (int)min((int64_t)a.tile, e_end - e0);
     const int tid = threadIdx.x;
     const int mode = a.mode;
 
@@ -2290,10 +2394,10 @@ k_interp_visc(const KArgs<real> a) {
     real *sM = sU + pad4(NE * G::template slots<PAD>() * V);
     real *sG = sM + pad4(NE * NSP * MS);
     const real *D1 = sOp, *Lm = sOp + N * N, *Lp = Lm + N;
-    const int64_t e0 = a.elem0 + (int64_t)blockIdx.x * NE;
+    const int64_t e0 = a.elem0 + (int64_t)blockIdx.x * a.tile;
     const int64_t e_end = a.elem0 + a.n_elem;
     if (e0 >= e_end) return;
-    const int ne = (int)min((int64_t)NE, e_end - e0);
+    const int ne = (int)min((int64_t)a.tile, e_end - e0);
     load_ops(a, sOp, N);
     load_state_rows<N, V, PAD>(sU, a.U, (const int32_t *)nullptr, e0, ne, NSP);
     load_tile(sM, a.MET, (const int32_t *)nullptr, e0, ne, NSP * MS);
@@ -2319,10 +2423,10 @@ k_interp(const KArgs<real> a) {
     real *sOp = reinterpret_cast<real *>(smem_raw);
     real *sU = sOp + ops_slots(N);
     const real *Lm = sOp + N * N, *Lp = Lm + N;
-    const int64_t e0 = a.elem0 + (int64_t)blockIdx.x * NE;
+    const int64_t e0 = a.elem0 + (int64_t)blockIdx.x * a.tile;
     const int64_t e_end = a.elem0 + a.n_elem;
     if (e0 >= e_end) return;
-    const int ne = (int)min((int64_t)NE, e_end - e0);
+    const int ne = (int)min((int64_t)a.tile, e_end - e0);
     load_ops(a, sOp, N);
     load_state_rows<N, V, false>(sU, a.U, (const int32_t *)nullptr, e0, ne, NSP);
     __syncthreads();
@@ -2963,10 +3067,34 @@ cudaError_t prep_smem(K kernel, size_t bytes) {
     return cudaSuccess;
 }
 
+// Elements per CTA of the tile kernels.  FP64 is bound by its FMA pipe (2
+// lanes per SM and clock), so a batch of fewer CTAs than SMs leaves most of
+// that pipe idle: 256 quads of p = 2 in 10 full tiles took 26 us per stage, in
+// 128 tiles of 2 elements 10.5 us.  The tile that leaves the busiest SM the
+// fewest warps of solution and flux points is taken, the largest of equals; at
+// full tiles the pipe is evenly loaded from some thousand elements on.  FP32
+// launches are latency-bound at such sizes and gain nothing.
+constexpr int kSMs = 152;
 template <int D, int N, typename real>
-cudaError_t launch_n(int kind, bool visc, const KArgs<real> &a, int grid_hint, cudaStream_t st) {
+int tile_elems(int64_t n_elem) {
     using G = Geo<D, N>;
-    const int64_t tiles = (a.n_elem + G::NE - 1) / G::NE;
+    if (sizeof(real) == 4) return G::NE;
+    int best = G::NE;
+    int64_t least = INT64_MAX;
+    for (int t = G::NE; t >= 1; --t) {
+        const int64_t ctas = (n_elem + t - 1) / t;
+        const int64_t warps = (ctas + kSMs - 1) / kSMs * ((t * G::NSP + 31) / 32 + (t * G::NFP + 31) / 32);
+        if (warps < least) { least = warps; best = t; }
+    }
+    return best;
+}
+
+template <int D, int N, typename real>
+cudaError_t launch_n(int kind, bool visc, const KArgs<real> &in, int grid_hint, cudaStream_t st) {
+    using G = Geo<D, N>;
+    KArgs<real> a = in;
+    a.tile = tile_elems<D, N, real>(a.n_elem);
+    const int64_t tiles = (a.n_elem + a.tile - 1) / a.tile;
     const bool ad = a.ADAPT != nullptr;   // adaptive steps: their own instantiation, register level 0
     const bool l1 = has_level1<N, real>() && a.regs_level == 1;
     const bool l2 = has_level1<N, real>() && a.regs_level == 2;

@@ -181,43 +181,7 @@ __device__ __forceinline__ void prim_line(const real *up, const LineRef<D, real>
     p = r.p + pp;
 }
 
-// viscous normal flux of the gradient Q for a state given by 1/rho, v and
-// specific energy Es; mi = mu / rho, ki = gamma mu / Pr / rho
-template <int D, typename real>
-__device__ __forceinline__ void visc_normal(const real (*Q)[D + 2], const real *v, real Es, real mi, real ki,
-                                            const real *n, real *out) {
-    constexpr int V = D + 2;
-    // rho times the velocity gradient [j][i] = d v_i / d x_j and, along n, the
-    // gradients of v and E
-    real gv[D][D], an[D], div = 0, qn0 = 0, qnE = 0;
-#pragma unroll
-    for (int j = 0; j < D; ++j) {
-#pragma unroll
-        for (int i = 0; i < D; ++i) gv[j][i] = Q[j][1 + i] - Q[j][0] * v[i];
-        div += gv[j][j];
-        qn0 += n[j] * Q[j][0];
-        qnE += n[j] * Q[j][V - 1];
-    }
-    real work = 0, va = 0;
-    const real d3 = real(2.0 / 3.0) * div;
-    out[0] = 0;
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-        real a = 0, b = 0;
-#pragma unroll
-        for (int j = 0; j < D; ++j) {
-            a += n[j] * gv[j][i];
-            b += n[j] * gv[i][j];
-        }
-        an[i] = a;
-        out[1 + i] = mi * (a + b - d3 * n[i]);
-        work += v[i] * out[1 + i];
-        va += v[i] * an[i];
-    }
-    out[V - 1] = work + ki * (qnE - qn0 * Es - va);
-}
-
-// the same for the rank-one gradient lf (x) dd (the lifting of a jump)
+// visc_normal for the rank-one gradient lf (x) dd (the lifting of a jump)
 template <int D, typename real>
 __device__ __forceinline__ void visc_lift(const real *lf, const real *dd, const real *v, real Es, real mi, real ki,
                                           const real *n, real *out) {
