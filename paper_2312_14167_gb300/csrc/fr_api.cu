@@ -34,6 +34,7 @@ cudaError_t prepare_2_f64(int N, bool visc);
 cudaError_t prepare_3_f32(int N, bool visc);
 cudaError_t prepare_3_f64(int N, bool visc);
 cudaError_t mortar_2_f32(const MArgs<float> &a, cudaStream_t s);
+cudaError_t mortar_line(const MortarLineArgs &a, cudaStream_t s);
 cudaError_t mortar_2_f64(const MArgs<double> &a, cudaStream_t s);
 cudaError_t mortar_3_f32(const MArgs<float> &a, cudaStream_t s);
 cudaError_t mortar_3_f64(const MArgs<double> &a, cudaStream_t s);
@@ -183,6 +184,12 @@ struct fr_solver {
     // one chunk's copy overlaps the previous chunk's conversion) and events
     cudaStream_t xfer = nullptr;
     cudaEvent_t xev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+    // independent launches of a captured step (degree groups, samples) become
+    // parallel branches of its graph: forked onto these streams
+    bool capturing = false;
+    static constexpr int kSide = 5;
+    cudaStream_t side[kSide] = {};
+    cudaEvent_t fork = nullptr, join[kSide] = {};
     std::string schedule_source = "default";
     double schedule_ms = 0.0;
     std::vector<std::unique_ptr<fr_mesh>> host_meshes;   // for probe location
@@ -203,6 +210,12 @@ namespace {
             return FR_ERR_CUDA;                                                    \
         }                                                                          \
     } while (0)
+
+// May the stages of this batch run as one fused kernel?  BR2 with conforming
+// faces only, or (2-D FP32, fixed steps: the line kernel) mortar faces too.
+bool fusable_batch(int dim, bool fp64, bool visc, bool adapt, const fr_config &cfg, int64_t n_mortar) {
+    return visc && cfg.viscous_scheme == FR_VISC_BR2 && (n_mortar == 0 || (dim == 2 && !fp64 && !adapt));
+}
 
 // propagate a failed fr_status
 #define FR_TRY(call)                      \
@@ -470,6 +483,7 @@ struct Launch {
     int64_t partial_slot = 0;     // first partial-sum block of the launch
     int64_t n_partials = 0;       // K_REDUCE: partial-sum blocks to reduce
     int grid = 1;
+    cudaStream_t stream = nullptr;   // null: the solver's
 };
 
 template <typename real>
@@ -495,12 +509,13 @@ cudaError_t do_launch(const fr_solver *s, const Launch &L) {
     if (L.n_partials > 0) a.n_partials = L.n_partials;
     const int N = s->grp[L.g].N;
     const bool visc = s->visc;
+    const cudaStream_t st = L.stream ? L.stream : s->stream;
     if constexpr (std::is_same<real, float>::value) {
-        return s->dim == 2 ? frk::launch_2_f32(N, L.kind, visc, a, L.grid, s->stream)
-                           : frk::launch_3_f32(N, L.kind, visc, a, L.grid, s->stream);
+        return s->dim == 2 ? frk::launch_2_f32(N, L.kind, visc, a, L.grid, st)
+                           : frk::launch_3_f32(N, L.kind, visc, a, L.grid, st);
     } else {
-        return s->dim == 2 ? frk::launch_2_f64(N, L.kind, visc, a, L.grid, s->stream)
-                           : frk::launch_3_f64(N, L.kind, visc, a, L.grid, s->stream);
+        return s->dim == 2 ? frk::launch_2_f64(N, L.kind, visc, a, L.grid, st)
+                           : frk::launch_3_f64(N, L.kind, visc, a, L.grid, st);
     }
 }
 
@@ -562,6 +577,44 @@ cudaError_t launch(const fr_solver *s, const Launch &L) {
     return timed(s, prof_kind(L), [&] { return s->fp64 ? do_launch<double>(s, L) : do_launch<float>(s, L); });
 }
 
+// Launches that neither read nor write what another of them writes (the
+// degree groups of one pass, the samples).  While a step is captured they
+// become parallel branches of the graph, so that the small launches of the
+// low-degree groups (8-11 us each at any size) run beside the large one.
+fr_status launch_all(fr_solver *s, std::vector<Launch> &ls, int64_t &cnt) {
+    const size_t extra = ls.size() > 1 ? std::min(ls.size() - 1, (size_t)fr_solver::kSide) : 0;
+    const bool fork = s->capturing && extra > 0;
+    if (fork) {
+        FR_CK(cudaEventRecord(s->fork, s->stream));
+        for (size_t i = 0; i < extra; ++i) {
+            ls[i + 1].stream = s->side[i];
+            FR_CK(cudaStreamWaitEvent(s->side[i], s->fork, 0));
+        }
+    }
+    for (const Launch &l : ls) {
+        FR_CK(launch(s, l));
+        ++cnt;
+    }
+    if (fork)
+        for (size_t i = 0; i < extra; ++i) {
+            FR_CK(cudaEventRecord(s->join[i], s->side[i]));
+            FR_CK(cudaStreamWaitEvent(s->stream, s->join[i], 0));
+        }
+    return FR_OK;
+}
+
+// the streams and events of launch_all, made before a capture begins
+cudaError_t ensure_side(fr_solver *s) {
+    if (s->fork) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < fr_solver::kSide && e == cudaSuccess; ++i) {
+        if (!s->side[i]) e = cudaStreamCreateWithFlags(&s->side[i], cudaStreamNonBlocking);
+        if (e == cudaSuccess && !s->join[i]) e = cudaEventCreateWithFlags(&s->join[i], cudaEventDisableTiming);
+    }
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming);
+    return e;
+}
+
 // mortar pass over the faces [m0, m0 + count) on face buffer parity par
 cudaError_t mortar(const fr_solver *s, int pass, int par, int64_t m0, int64_t count) {
     if (count <= 0) return cudaSuccess;
@@ -570,13 +623,42 @@ cudaError_t mortar(const fr_solver *s, int pass, int par, int64_t m0, int64_t co
     });
 }
 
+// inbound gradient-flux-part buffer of face parity par (fused stage)
+char *fvbuf(const Group &G, int par) { return par == 0 ? G.FV : G.FV2; }
+
+// after the traces of face-buffer parity par have been written: what the next
+// evaluation needs of the mortar faces [m0, m0 + count) (the carried traces;
+// line kernels: and the common fluxes)
+cudaError_t mortar_traces(const fr_solver *s, int par, int64_t m0, int64_t count) {
+    if (count <= 0) return cudaSuccess;
+    if (!s->fused) return mortar(s, 0, par, m0, count);
+    return timed(s, P_OTHER, [&] {
+        frk::MortarLineArgs a;
+        std::memset(&a, 0, sizeof(a));
+        for (size_t g = 0; g < s->grp.size(); ++g) {
+            const Group &G = s->grp[g];
+            a.UF[g] = (float *)G.UF[par];
+            a.FV[g] = (const float *)fvbuf(G, par);
+            a.FGEO[g] = (const float *)G.FGEO;
+            a.MFLUX[g] = (float *)G.MFLUX;
+            a.fp_real[g] = G.fp_real;
+        }
+        a.faces = s->MORT + m0;
+        a.n_faces = count;
+        a.mats = (const float *)s->MATS;
+        a.gamma = (float)s->cfg.gamma;
+        a.mu = (float)s->cfg.mu;
+        a.kq = (float)(s->cfg.mu * s->cfg.gamma / (s->cfg.prandtl > 0 ? s->cfg.prandtl : 1.0));
+        a.flux = s->cfg.flux;
+        a.ref = s->ref32;
+        return frk::mortar_line(a, s->stream);
+    });
+}
+
 int grid_for(int64_t items) {
     int64_t g = (items + 255) / 256;
     return (int)std::max<int64_t>(1, std::min<int64_t>(g, kPartialBlocks));
 }
-
-// inbound gradient-flux-part buffer of face parity par (fused stage)
-char *fvbuf(const Group &G, int par) { return par == 0 ? G.FV : G.FV2; }
 
 // One stage evaluation reading face-buffer parity par (and writing par ^ 1):
 // [gradient kernels,] mortar common fluxes, stage kernels with RK mode
@@ -585,21 +667,23 @@ char *fvbuf(const Group &G, int par) { return par == 0 ? G.FV : G.FV2; }
 fr_status enqueue_eval(fr_solver *s, int par, int mode, double rk_a, double rk_b, double rk_c, int64_t &cnt) {
     const int G = (int)s->grp.size();
     if (s->visc && !s->fused) {
-        for (int g = 0; g < G; ++g) {
+        std::vector<Launch> ls;
+        for (int g = G - 1; g >= 0; --g) {
             Launch l;
             l.kind = frk::K_GRAD;
             l.g = g;
             l.n_elem = s->grp[g].E;
             l.UFin = s->grp[g].UF[par];
-            FR_CK(launch(s, l));
-            ++cnt;
+            ls.push_back(l);
         }
+        FR_TRY(launch_all(s, ls, cnt));
     }
-    if (s->n_mortar > 0) {
+    if (s->n_mortar > 0 && !s->fused) {
         FR_CK(mortar(s, 1, par, 0, s->n_mortar));
         ++cnt;
     }
-    for (int g = 0; g < G; ++g) {
+    std::vector<Launch> fs;
+    for (int g = G - 1; g >= 0; --g) {
         Launch f;
         f.kind = s->fused ? frk::K_STAGE : frk::K_FLUX;
         f.g = g;
@@ -612,11 +696,11 @@ fr_status enqueue_eval(fr_solver *s, int par, int mode, double rk_a, double rk_b
         f.rk_a = rk_a;
         f.rk_b = rk_b;
         f.rk_c = rk_c;
-        FR_CK(launch(s, f));
-        ++cnt;
+        fs.push_back(f);
     }
+    FR_TRY(launch_all(s, fs, cnt));
     if (s->n_mortar > 0 && mode != frk::M_BS_START && mode != frk::M_BS_4) {
-        FR_CK(mortar(s, 0, par ^ 1, 0, s->n_mortar));
+        FR_CK(mortar_traces(s, par ^ 1, 0, s->n_mortar));
         ++cnt;
     }
     return FR_OK;
@@ -626,14 +710,7 @@ fr_status enqueue_eval(fr_solver *s, int par, int mode, double rk_a, double rk_b
 // faces of the step's final state).
 fr_status enqueue_samples(fr_solver *s, int par, int64_t &cnt) {
     const int G = (int)s->grp.size();
-    for (int g = 0; g < G; ++g) {
-        if (s->grp[g].n_probe <= 0) continue;
-        Launch pr;
-        pr.kind = frk::K_PROBE;
-        pr.g = g;
-        FR_CK(launch(s, pr));
-        ++cnt;
-    }
+    std::vector<Launch> ls;
     for (int g = 0; g < G; ++g) {
         if (s->grp[g].n_wall <= 0) continue;
         Launch fo;
@@ -643,10 +720,16 @@ fr_status enqueue_samples(fr_solver *s, int par, int64_t &cnt) {
         fo.elist = s->grp[g].WALL;
         fo.n_elem = s->grp[g].n_wall;
         fo.UFin = s->grp[g].UF[par];
-        FR_CK(launch(s, fo));
-        ++cnt;
+        ls.push_back(fo);
     }
-    return FR_OK;
+    for (int g = 0; g < G; ++g) {
+        if (s->grp[g].n_probe <= 0) continue;
+        Launch pr;
+        pr.kind = frk::K_PROBE;
+        pr.g = g;
+        ls.push_back(pr);
+    }
+    return launch_all(s, ls, cnt);
 }
 
 // Face-buffer parity flips of one step (one per stage evaluation).
@@ -657,19 +740,20 @@ int step_flips(const fr_solver *s) {
 // Face states (and, fused BR2, gradient flux parts) of the current state U
 // of every instance into face-buffer parity par, mortar traces included.
 fr_status enqueue_faces(fr_solver *s, int par, int64_t &cnt) {
-    for (size_t g = 0; g < s->grp.size(); ++g) {
+    std::vector<Launch> ls;
+    for (int g = (int)s->grp.size() - 1; g >= 0; --g) {
         const Group &G = s->grp[g];
         Launch in;
         in.kind = s->fused ? frk::K_INTERP_VISC : frk::K_INTERP;
-        in.g = (int)g;
+        in.g = g;
         in.n_elem = G.E;
         in.UFout = G.UF[par];
         in.FVout = fvbuf(G, par);
-        FR_CK(launch(s, in));
-        ++cnt;
+        ls.push_back(in);
     }
+    FR_TRY(launch_all(s, ls, cnt));
     if (s->n_mortar > 0) {
-        FR_CK(mortar(s, 0, par, 0, s->n_mortar));
+        FR_CK(mortar_traces(s, par, 0, s->n_mortar));
         ++cnt;
     }
     return FR_OK;
@@ -800,7 +884,7 @@ fr_status residual_into_res(fr_solver *s, int inst, int mode) {
             FR_CK(launch(s, l));
         }
     }
-    FR_CK(mortar(s, 1, s->parity, s->moff[inst], s->mcnt[inst]));
+    if (!s->fused) FR_CK(mortar(s, 1, s->parity, s->moff[inst], s->mcnt[inst]));
     for (int g = 0; g < G; ++g) {
         Launch f;
         f.kind = s->fused ? frk::K_STAGE : frk::K_FLUX;
@@ -1310,9 +1394,9 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
     // on 31,722 quads, 3.3 against 5.9 on 48^3 hexes of p = 3, 4.7 against 6.8
     // on 57,120 of p = 4); elsewhere and for adaptive steps the pair is, and
     // fr_tune measures both
-    const bool fusable = s->visc && cfg->viscous_scheme == FR_VISC_BR2 && P.n_mortar == 0;
+    const bool fusable = fusable_batch(dim, s->fp64, s->visc, s->adapt, *cfg, P.n_mortar);
     s->fused = fusable && !s->fp64 && !s->adapt;
-    for (int g = 0; g < P.G; ++g) s->fused = s->fused && s->grp[g].N >= 2;
+    for (int g = 0; g < P.G; ++g) s->fused = s->fused && (dim == 2 || s->grp[g].N >= 2);
     if (fusable) {
         // partner lifting coefficients per own flux point (FP64, then cast):
         // lf = sum_m l_m(side) g'_side(m) (1/J) S[k][:] along the partner's line
@@ -1335,7 +1419,7 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
 #pragma omp parallel for schedule(static)
             for (int64_t q = 0; q < G.E * nfp; ++q) {
                 const int32_t pt = part[g][q];
-                if (pt < 0) continue;
+                if (pt < 0 || pt >= G.fp_real) continue;
                 for (int jd = 0; jd < dim; ++jd) lfp[q * dim + jd] = lf[(size_t)pt * dim + jd];
             }
             FR_CK(up_real(G.LFP, lfp, lfp.size()));
@@ -1437,6 +1521,11 @@ extern "C" void fr_solver_destroy(fr_solver *s) {
     }
     for (cudaEvent_t e : s->xev)
         if (e) cudaEventDestroy(e);
+    for (cudaEvent_t e : s->join)
+        if (e) cudaEventDestroy(e);
+    if (s->fork) cudaEventDestroy(s->fork);
+    for (cudaStream_t st : s->side)
+        if (st) cudaStreamDestroy(st);
     delete s;
 }
 
@@ -1499,7 +1588,7 @@ fr_status enqueue_upload(fr_solver *s, int inst, const double *u, std::vector<do
         in.FVout = fvbuf(G, s->parity);
         FR_CK(launch(s, in));
     }
-    FR_CK(mortar(s, 0, s->parity, s->moff[inst], s->mcnt[inst]));
+    FR_CK(mortar_traces(s, s->parity, s->moff[inst], s->mcnt[inst]));
     return FR_OK;
 }
 
@@ -1816,9 +1905,12 @@ extern "C" fr_status fr_rk_step(fr_solver *s, int n_steps) {
         if (s->stream) {
             if (!s->graph[p0]) {
                 cudaGraph_t g;
+                FR_CK(ensure_side(s));
                 FR_CK(cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal));
                 int64_t cnt = 0;
+                s->capturing = true;
                 fr_status st = enqueue_step(s, p0, &cnt);
+                s->capturing = false;
                 cudaError_t ce = cudaStreamEndCapture(s->stream, &g);
                 if (st != FR_OK) return st;
                 FR_CK(ce);
@@ -2406,8 +2498,8 @@ bool apply_schedule(fr_solver *s, const std::string &v, const char *source) {
     const size_t r = v.find("regs=");
     const int regs = r == std::string::npos ? 0 : std::atoi(v.c_str() + r + 5);
     const bool tc = v.find("contract=tc") != std::string::npos;
-    const bool fusable = s->visc && s->cfg.viscous_scheme == FR_VISC_BR2 && s->n_mortar == 0;
-    if ((fused && !fusable) || regs < 0 || regs >= frk::kRegLevels || (tc && s->fp64)) return false;
+    const bool fusable = fusable_batch(s->dim, s->fp64, s->visc, s->adapt, s->cfg, s->n_mortar);
+    if ((fused && (!fusable || (tc && s->n_mortar > 0))) || regs < 0 || regs >= frk::kRegLevels || (tc && s->fp64)) return false;
     s->fused = fused;
     // FP64 and adaptive steps run the stage kernels at register level 0 only
     s->regs_level = (s->fp64 || s->adapt) ? 0 : regs;
@@ -2456,9 +2548,9 @@ extern "C" fr_status fr_tune(fr_solver *s, const char *cache_path, int mode, cha
     // candidates: stage schedule x register level
     struct Cand { bool fused; int regs; bool tc; double ms; };
     std::vector<Cand> cands;
-    const bool fusable = s->visc && s->cfg.viscous_scheme == FR_VISC_BR2 && s->n_mortar == 0;
+    const bool fusable = fusable_batch(s->dim, s->fp64, s->visc, s->adapt, s->cfg, s->n_mortar);
     for (int c = 0; c < (s->fp64 ? 1 : 2); ++c)
-        for (int f = 0; f < (fusable ? 2 : 1); ++f)
+        for (int f = 0; f < (fusable && !(c == 1 && s->n_mortar > 0) ? 2 : 1); ++f)
             for (int r = 0; r < ((s->fp64 || s->adapt) ? 1 : frk::kRegLevels); ++r) cands.push_back({f == 1, r, c == 1, 0.0});
     const int warm = 2, timed = 3;
     const int flips = step_flips(s);
@@ -2502,7 +2594,7 @@ extern "C" fr_status fr_tune(fr_solver *s, const char *cache_path, int mode, cha
                 in.FVout = fvbuf(G, s->parity);
                 if (launch(s, in) != cudaSuccess) st = FR_ERR_CUDA;
             }
-            if (st == FR_OK && mortar(s, 0, s->parity, s->moff[i], s->mcnt[i]) != cudaSuccess) st = FR_ERR_CUDA;
+            if (st == FR_OK && mortar_traces(s, s->parity, s->moff[i], s->mcnt[i]) != cudaSuccess) st = FR_ERR_CUDA;
         }
         if (st == FR_OK) st = bs_start_if_needed(s);
         for (int it = 0; it < warm + timed && st == FR_OK; ++it) {

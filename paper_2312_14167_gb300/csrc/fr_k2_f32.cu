@@ -63,6 +63,12 @@ cudaError_t prepare_2_f32(int N, bool visc) {
     }
 }
 
+cudaError_t mortar_line(const MortarLineArgs &a, cudaStream_t s) {
+    if (a.n_faces <= 0) return cudaSuccess;
+    k_mortar_line<<<(unsigned)((a.n_faces + 15) / 16), 128, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
 cudaError_t mortar_2_f32(const MArgs<float> &a, cudaStream_t s) {
     return launch_mortar<2, float>(a, s);
 }

@@ -2411,6 +2411,10 @@ k_interp_visc(const KArgs<real> a) {
 #include "fr_line.cuh"
 namespace frk {
 
+// does this launch use a line kernel?
+template <int D, int N, typename real>
+__host__ __device__ constexpr bool has_line() { return sizeof(real) == 4 && (D == 2 || N >= 2); }
+
 // --------------------------------------------------------------------------
 // K_INTERP: face values of the current state (after fr_set_state)
 // --------------------------------------------------------------------------
@@ -3021,6 +3025,99 @@ __global__ void __launch_bounds__(128) k_mortar(const MArgs<real> a) {
         real *dst = a.MFLUX[F.glo] + (F.lo_box - a.fp_real[F.glo] + lane) * V;
 #pragma unroll
         for (int v = 0; v < V; ++v) dst[v] = -acc[v];
+    }
+}
+
+static __global__ void __launch_bounds__(128) k_mortar_line(const MortarLineArgs a) {
+    constexpr int D = 2, V = 4, MF = 16, MP = 5;
+    __shared__ float sLo[MF][MP][V], sHi[MF][MP][V], sFl[MF][MP][V], sFs[MF][MP][V];
+    const int q = threadIdx.x & 7, w = threadIdx.x >> 3;
+    const int64_t m = (int64_t)blockIdx.x * MF + w;
+    const bool face = m < a.n_faces;
+    const MortarFace F = a.faces[face ? m : a.n_faces - 1];
+    const bool lo = face && q < F.nlo, hi = face && q < F.nhi;
+    const float *T = a.mats + F.mat, *P = T + F.nhi * F.nlo;
+    // flux point r of a group: normal and own lifting coefficients
+    auto geo = [&](int g, int64_t r, int nf, float *n, float *lf) {
+        const float4 A = __ldg(reinterpret_cast<const float4 *>(a.FGEO[g]) + r / nf * (2 * nf) + r % nf);
+        n[0] = A.x; n[1] = A.y; lf[0] = A.z; lf[1] = A.w;
+    };
+    // own viscous normal flux: gradient part fv plus the lifting of the jump to uR
+    auto own_flux = [&](const float *u, const float *uR, const float *n, const float *lf, const float *fv, float *o) {
+        float full[V], dd[V], vel[D];
+        add_ref<V>(a.ref, u, full);
+        const float ir = 1.0f / full[0];
+#pragma unroll
+        for (int d = 0; d < D; ++d) vel[d] = full[1 + d] * ir;
+#pragma unroll
+        for (int v = 0; v < V; ++v) dd[v] = 0.5f * (uR[v] - u[v]);
+        visc_lift<D>(lf, dd, vel, full[V - 1] * ir, a.mu * ir, a.kq * ir, n, o);
+#pragma unroll
+        for (int v = 0; v < V; ++v) o[v] += fv[v];
+    };
+    float uh[V], ul[V], fvh[V], fvl[V];
+    if (hi) {
+        ld_v<V>(a.UF[F.ghi] + (F.hi_box + q) * V, uh);
+        ldg_v<V>(a.FV[F.ghi] + (F.hi_box + q) * V, fvh);
+#pragma unroll
+        for (int v = 0; v < V; ++v) sHi[w][q][v] = uh[v];
+    }
+    if (lo) {
+        ld_v<V>(a.UF[F.glo] + (F.lo_box + q) * V, ul);
+        ldg_v<V>(a.FV[F.glo] + (F.lo_box + q) * V, fvl);
+#pragma unroll
+        for (int v = 0; v < V; ++v) sLo[w][q][v] = ul[v];
+    }
+    __syncwarp();
+    float uRh[V] = {0, 0, 0, 0};
+    if (hi) {
+        for (int i = 0; i < F.nlo; ++i) {
+            const float t = T[q * F.nlo + i];
+#pragma unroll
+            for (int v = 0; v < V; ++v) uRh[v] += t * sLo[w][i][v];
+        }
+        st_v<V>(a.UF[F.ghi] + (F.hi_fp + q) * V, uRh);
+    }
+    if (lo) {
+        float uRl[V] = {0, 0, 0, 0}, n[D], lf[D], o[V];
+        for (int i = 0; i < F.nhi; ++i) {
+            const float t = P[q * F.nhi + i];
+#pragma unroll
+            for (int v = 0; v < V; ++v) uRl[v] += t * sHi[w][i][v];
+        }
+        st_v<V>(a.UF[F.glo] + (F.lo_fp + q) * V, uRl);
+        geo(F.glo, F.lo_fp + q, F.nlo, n, lf);
+        own_flux(ul, uRl, n, lf, fvl, o);
+#pragma unroll
+        for (int v = 0; v < V; ++v) sFl[w][q][v] = o[v];
+    }
+    __syncwarp();
+    if (hi) {
+        float n[D], lf[D], o[V], Fs[V], fl[V] = {0, 0, 0, 0};
+        geo(F.ghi, F.hi_fp + q, F.nhi, n, lf);
+        common_inviscid_pert<D>(a.flux, uh, uRh, n, a.ref, a.gamma, Fs);
+        own_flux(uh, uRh, n, lf, fvh, o);
+        for (int i = 0; i < F.nlo; ++i) {
+            const float t = T[q * F.nlo + i];
+#pragma unroll
+            for (int v = 0; v < V; ++v) fl[v] += t * sFl[w][i][v];
+        }
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            Fs[v] -= 0.5f * (o[v] - fl[v]);
+            sFs[w][q][v] = Fs[v];
+        }
+        st_v<V>(a.MFLUX[F.ghi] + (F.hi_box - a.fp_real[F.ghi] + q) * V, Fs);
+    }
+    __syncwarp();
+    if (lo) {
+        float o[V] = {0, 0, 0, 0};
+        for (int i = 0; i < F.nhi; ++i) {
+            const float t = P[q * F.nhi + i];
+#pragma unroll
+            for (int v = 0; v < V; ++v) o[v] -= t * sFs[w][i][v];
+        }
+        st_v<V>(a.MFLUX[F.glo] + (F.lo_box - a.fp_real[F.glo] + q) * V, o);
     }
 }
 

@@ -214,6 +214,19 @@ __device__ __forceinline__ void line_face(const KArgs<real> &a, const LineRef<D,
     constexpr int V = D + 2;
     const real gm1 = a.gamma - real(1);
     const bool inner = g.pt >= 0;
+    if (inner && g.pt >= (int32_t)a.fp_real) {
+        // mortar point: the common flux was formed on the mortar, relative to
+        // n . F(u_r); take n . (F(u_c) - F(u_r)) off
+        real Fc[V], vn, c2;
+        ldg_v<V>(a.MFLUX + (int64_t)(g.pt - (int32_t)a.fp_real) * V, Fs);
+        flux_normal_pert<D>(R.du, g.n, a.ref, gm1, a.gamma, Fc, vn, c2);
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            Fs[v] -= Fc[v];
+            dd[v] = real(0.5) * (uR[v] - uL[v]);
+        }
+        return;
+    }
     real uLl[V], uRl[V], ub[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) uLl[v] = uL[v] - R.du[v];
@@ -1318,8 +1331,28 @@ k_line3(const __grid_constant__ KArgs<float> a) {
     }
 }
 
-// does this launch use the line kernel?
-template <int D, int N, typename real>
-__host__ __device__ constexpr bool has_line() { return sizeof(real) == 4 && N >= 2; }
+// --------------------------------------------------------------------------
+// Mortar faces of 2-D line-kernel batches, once per stage, after the line
+// kernels have put every mortar side's trace and gradient flux part into its
+// outbox rows.  Eight lanes per face: carry the traces across (T, P; see
+// K_MORTAR), then form the common flux of the next stage on the mortar: both
+// sides' own viscous normal fluxes are their gradient part plus the lifting of
+// their jump, the lower side's carried by T; the lower side takes minus the
+// projection of the common flux.  (The gradient + flux pair needs two mortar
+// launches per stage, around the flux kernel.)
+// --------------------------------------------------------------------------
+struct MortarLineArgs {
+    float *UF[5];                  // face states of the pass, per degree group
+    const float *FV[5];            // gradient flux parts of the pass
+    const float *FGEO[5];
+    float *MFLUX[5];
+    int64_t fp_real[5];
+    const struct MortarFace *faces;
+    int64_t n_faces;
+    const float *mats;
+    float gamma, mu, kq;
+    int flux;
+    RefState<float> ref;
+};
 
 }  // namespace frk

@@ -62,3 +62,26 @@ def test_steps_follow_the_oracle(shape, p, rk):
     for _ in range(5):
         u = step(disc.residual, u, case.dt)
     assert FC.rel_l2(sol.get_state(0), u) < 1e-6
+
+
+@pytest.mark.parametrize("flux", ["rusanov", "roe"])
+@pytest.mark.parametrize("degrees", [(0, 1, 2, 3), (1, 4), (0, 4), (2, 3)])
+def test_mortar_faces(degrees, flux):
+    """Several degrees in one mesh: every degree group's line kernel and the
+    mortar faces between them (most faces here), residual and steps."""
+    from oracle.fr_var import VarFRDiscretisation
+    from paper_2312_14167_gb300 import fr
+    case = _case((11, 7), 3, flux=flux)
+    mesh = case.meshes[0]
+    ep = M.checker_degrees(mesh, degrees, seed=3)
+    disc = VarFRDiscretisation(mesh, ep, FC.oracle_disc(case).phys)
+    sol = fr.Solver([fr.Mesh(mesh, ep)], FC.lib_config(case, "fp32"))
+    assert "stage=fused" in sol.schedule()[0]
+    u = FC.initial_state(case, disc.sol_coords())
+    sol.set_state(0, u)
+    ref = disc.residual(FC.fp32_input(case, u))
+    assert FC.rel_l2(sol.residual(0), ref) < 1e-5
+    sol.rk_step(5)
+    for _ in range(5):
+        u = T.lsrk45_step(disc.residual, u, case.dt)
+    assert FC.rel_l2(sol.get_state(0), u) < 1e-6
