@@ -216,11 +216,10 @@ fr_status fr_set_state(fr_solver *solver, int inst, const double *u);
 fr_status fr_get_state(fr_solver *solver, int inst, double *u);
 /* The states of all instances at once: u holds instance 0's state, then
  * instance 1's, ... (each in the layout of fr_set_state), sum over instances
- * of n_sol_points * V doubles.  When every instance lies in one degree group
- * (the usual case) the whole batch moves in one copy each way through the
- * workspace's FP64 staging area, converted by one launch per run of
- * consecutive instances; an instance with elements of several degrees goes
- * through a host reorder, one instance after another.  The stream is
+ * of n_sol_points * V doubles.  The whole batch moves in one copy each way
+ * through the workspace's FP64 staging area, converted by one launch per run
+ * of consecutive instances (instances with elements of several degrees: per
+ * degree, each element at its own place in the staging area).  The stream is
  * synchronised once, which is what a poll evaluator that moves every
  * candidate each step wants; with pinned host memory the copies run at the
  * host link's speed.  Same results as one fr_set_state / fr_get_state per

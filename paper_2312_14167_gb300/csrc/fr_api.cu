@@ -99,6 +99,7 @@ struct Group {
     char *R3 = nullptr;
     int64_t ebase = 0;
     int32_t *PART = nullptr, *EINST = nullptr, *WALL = nullptr;
+    int64_t *EOFF = nullptr;   // batches with spread instances: every element's place in the host order
     bool use_divref = false;   // FP32: the reference flux has a residual here
     int n_probe = 0;
     RefElem ref;
@@ -112,6 +113,7 @@ struct Plan {
     int64_t E[frk::kMaxGroups] = {}, n_wall[frk::kMaxGroups] = {};
     int64_t box_lo[frk::kMaxGroups] = {}, box_hi[frk::kMaxGroups] = {};
     int64_t nb = 0, stage_doubles = 0, n_mortar = 0;
+    bool spread = false;   // some instance has elements in several groups
     std::map<int, int64_t> mat_off;   // (p_lo, p_hi, orient) -> offset in the matrix table
     int64_t mat_reals = 0;
 };
@@ -124,6 +126,7 @@ struct fr_solver {
     int dim = 0, n_inst = 0, V = 0, MS = 0;
     fr_config cfg{};
     bool fp64 = true, visc = false;
+    bool mapped = false;   // some instance is spread over several groups: conversions use EOFF
     std::vector<fr::Group> grp;
     int64_t nb = 0;
     cudaStream_t stream = nullptr;
@@ -278,6 +281,7 @@ Plan make_plan(fr_mesh *const *meshes, int n_inst) {
     for (int i = 0; i < n_inst; ++i) {
         const fr_mesh *m = meshes[i];
         int64_t nsp_inst = 0;
+        P.spread = P.spread || !m->parts.empty();
         for (const fr_mesh *pm : parts_of(m)) {
             const int g = P.group_of_degree[pm->p];
             const int nfp = pm->ref.nfp;
@@ -310,7 +314,7 @@ Plan make_plan(fr_mesh *const *meshes, int n_inst) {
 }
 
 struct GroupLayout {
-    size_t U, R1, R2, RES, UF0, UF1, FV, MET, NRM, MFLUX, PART, EINST, WALL, DIVREF, FV2, LFP, R3, FGEO, METL;
+    size_t U, R1, R2, RES, UF0, UF1, FV, MET, NRM, MFLUX, PART, EINST, WALL, DIVREF, FV2, LFP, R3, FGEO, METL, EOFF;
 };
 struct Layout {
     GroupLayout g[frk::kMaxGroups];
@@ -348,6 +352,7 @@ Layout make_layout(const Plan &P, int n_inst, bool fp64, bool visc, bool adapt) 
         G.LFP = take(visc ? (size_t)E * nfp * dim * rs : 16);
         G.R3 = take(adapt ? st : 16);
         G.FGEO = take(visc && !fp64 ? (size_t)E * nfp * frk::face_geo(dim) * 4 : 16);
+        G.EOFF = take(P.spread ? (size_t)E * 8 : 16);
         G.METL = take(visc && !fp64 && dim == 3 ? (size_t)E * nsp * MS * 4 : 16);
     }
     L.BTAG = take((size_t)P.nb * 4);
@@ -421,6 +426,7 @@ void fill_args(const fr_solver *s, int g, frk::KArgs<real> &a) {
     a.LFP = (const real *)G.LFP;
     a.FGEO = (const float *)G.FGEO;
     a.METL = (const float *)G.METL;
+    a.EOFF = s->mapped ? G.EOFF : nullptr;
     a.kq = (real)((s->visc ? s->cfg.mu : 0.0) * s->cfg.gamma / (s->cfg.prandtl > 0 ? s->cfg.prandtl : 1.0));
     a.local_ref = s->local_ref ? 1 : 0;
     a.regs_level = s->regs_level;
@@ -932,10 +938,11 @@ fr_status reduce_integral(fr_solver *s, int inst, int src, double *out_sums, dou
 // instance spread over several groups?
 bool spread(const fr_solver *s, int inst) { return !s->egroup[inst].empty(); }
 
-// staging offset (doubles) of group g's block for one instance
-int64_t stage_block(const fr_solver *s, int inst, int g) {
+// offset (doubles) of an instance in the FP64 staging buffer, which holds the
+// batch in the host's order
+int64_t stage_begin(const fr_solver *s, int inst) {
     int64_t o = 0;
-    for (int h = 0; h < g; ++h) o += s->grp[h].ne[inst] * s->grp[h].nsp * s->V;
+    for (int i = 0; i < inst; ++i) o += s->inst_nsp[i] * s->V;
     return o;
 }
 
@@ -1132,6 +1139,7 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
     s->stream = (cudaStream_t)stream;
     s->nb = P.nb;
     s->n_mortar = P.n_mortar;
+    s->mapped = P.spread;
     s->grp.resize(P.G);
     for (int g = 0; g < P.G; ++g) {
         Group &G = s->grp[g];
@@ -1171,6 +1179,7 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
         G.R3 = w + gl.R3;
         G.FGEO = w + gl.FGEO;
         G.METL = w + gl.METL;
+        G.EOFF = (int64_t *)(w + gl.EOFF);
     }
     s->BTAG = (int32_t *)(w + L.BTAG); s->BVREF = w + L.BVREF;
     s->stage64 = (double *)(w + L.STAGE);
@@ -1225,6 +1234,22 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
             s->elocal[i][e] = m->local[e];
             s->esp[i][e] = o;
             o += pm->ref.nsp;
+        }
+    }
+
+    std::vector<std::vector<int64_t>> eoff(P.G);
+    if (s->mapped) {
+        // place of every element in the batch's host order (doubles)
+        for (int g = 0; g < P.G; ++g) eoff[g].resize(s->grp[g].E);
+        int64_t at = 0;
+        for (int i = 0; i < n_inst; ++i) {
+            for (int g = 0; g < P.G; ++g)
+                if (!spread(s.get(), i))
+                    for (int64_t e = 0; e < s->grp[g].ne[i]; ++e)
+                        eoff[g][s->grp[g].off[i] + e] = at + e * s->grp[g].nsp * s->V;
+            for (size_t e = 0; e < s->egroup[i].size(); ++e)
+                eoff[s->egroup[i][e]][s->grp[s->egroup[i][e]].off[i] + s->elocal[i][e]] = at + s->esp[i][e] * s->V;
+            at += s->inst_nsp[i] * s->V;
         }
     }
 
@@ -1373,6 +1398,7 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
         FR_CK(up(G.PART, part[g].data(), part[g].size() * 4));
         FR_CK(up(G.EINST, einst[g].data(), einst[g].size() * 4));
         FR_CK(up(G.WALL, wall[g].data(), wall[g].size() * 4));
+        FR_CK(up(G.EOFF, eoff[g].data(), eoff[g].size() * 8));
         const size_t st_bytes = (size_t)G.E * G.nsp * s->V * s->rsz;
         const size_t fc_bytes = ((size_t)G.E * G.nfp + G.n_box) * s->V * s->rsz;
         FR_CK(cudaMemsetAsync(G.U, 0, st_bytes, cs));
@@ -1545,40 +1571,34 @@ fr_status reset_step_control(fr_solver *s, int inst) {
     return FR_OK;
 }
 
+// Conversion (K_TO_REAL or K_TO_F64, src: 0 state, 1 residual) between the
+// staging buffer and elements [e0, e0 + ne) of group g; so: their staging
+// offset (mapped batches find every element's own)
+fr_status convert(fr_solver *s, int kind, int src, int g, int64_t e0, int64_t ne, int64_t so) {
+    Launch c;
+    c.kind = kind;
+    c.g = g;
+    c.elem0 = e0;
+    c.n_elem = ne;
+    c.integral_src = src;
+    c.stage_off = s->mapped ? 0 : so;
+    c.grid = grid_for(ne * s->grp[g].nsp * s->V);
+    FR_CK(launch(s, c));
+    return FR_OK;
+}
+
 // Enqueue the upload of one instance's FP64 host state (the ABI's element
-// order) and the derivation of its face values; no synchronisation.  An
-// instance spread over several degree groups is reordered on the host into
-// `tmp`, which must stay alive until the stream has been synchronised.
-fr_status enqueue_upload(fr_solver *s, int inst, const double *u, std::vector<double> &tmp) {
+// order) and the derivation of its face values; no synchronisation.
+fr_status enqueue_upload(fr_solver *s, int inst, const double *u) {
     const int V = s->V;
     FR_CK(cudaMemsetAsync(s->FLAGS + inst, 0, 4, s->stream));
     if (s->adapt) FR_TRY(reset_step_control(s, inst));
-    const size_t n = (size_t)s->inst_nsp[inst] * V;
-    if (!spread(s, inst)) {
-        FR_CK(cudaMemcpyAsync(s->stage64, u, n * 8, cudaMemcpyHostToDevice, s->stream));
-    } else {
-        // host reorder: element order -> group blocks
-        tmp.resize(n);
-        std::vector<int64_t> blk(s->grp.size());
-        for (size_t g = 0; g < s->grp.size(); ++g) blk[g] = stage_block(s, inst, (int)g);
-        for (size_t e = 0; e < s->egroup[inst].size(); ++e) {
-            const int g = s->egroup[inst][e];
-            const size_t cnt = (size_t)s->grp[g].nsp * V;
-            std::memcpy(&tmp[blk[g] + s->elocal[inst][e] * cnt], u + s->esp[inst][e] * V, cnt * 8);
-        }
-        FR_CK(cudaMemcpyAsync(s->stage64, tmp.data(), n * 8, cudaMemcpyHostToDevice, s->stream));
-    }
+    const int64_t so = stage_begin(s, inst);
+    FR_CK(cudaMemcpyAsync(s->stage64 + so, u, (size_t)s->inst_nsp[inst] * V * 8, cudaMemcpyHostToDevice, s->stream));
     for (size_t g = 0; g < s->grp.size(); ++g) {
         const Group &G = s->grp[g];
         if (G.ne[inst] <= 0) continue;
-        Launch c;
-        c.kind = frk::K_TO_REAL;
-        c.g = (int)g;
-        c.elem0 = G.off[inst];
-        c.n_elem = G.ne[inst];
-        c.stage_off = stage_block(s, inst, (int)g);
-        c.grid = grid_for(G.ne[inst] * G.nsp * V);
-        FR_CK(launch(s, c));
+        FR_TRY(convert(s, frk::K_TO_REAL, 0, (int)g, G.off[inst], G.ne[inst], so));
         Launch in;
         in.kind = s->fused ? frk::K_INTERP_VISC : frk::K_INTERP;
         in.g = (int)g;
@@ -1593,62 +1613,38 @@ fr_status enqueue_upload(fr_solver *s, int inst, const double *u, std::vector<do
 }
 
 // Enqueue the FP64 conversion of one instance's state (src 0) or residual
-// (src 1) and its download to u; no synchronisation.  An instance spread over
-// several degree groups lands in `tmp` and is put in element order by
-// finish_download once the stream has been synchronised.
-fr_status enqueue_download(fr_solver *s, int inst, int src, double *u, std::vector<double> &tmp) {
-    const int V = s->V;
-    const size_t n = (size_t)s->inst_nsp[inst] * V;
+// (src 1) and its download to u; no synchronisation.
+fr_status enqueue_download(fr_solver *s, int inst, int src, double *u) {
+    const int64_t so = stage_begin(s, inst);
     for (size_t g = 0; g < s->grp.size(); ++g) {
         const Group &G = s->grp[g];
-        if (G.ne[inst] <= 0) continue;
-        Launch c;
-        c.kind = frk::K_TO_F64;
-        c.g = (int)g;
-        c.elem0 = G.off[inst];
-        c.n_elem = G.ne[inst];
-        c.integral_src = src;
-        c.stage_off = stage_block(s, inst, (int)g);
-        c.grid = grid_for(G.ne[inst] * G.nsp * V);
-        FR_CK(launch(s, c));
+        if (G.ne[inst] > 0) FR_TRY(convert(s, frk::K_TO_F64, src, (int)g, G.off[inst], G.ne[inst], so));
     }
-    if (!spread(s, inst)) {
-        FR_CK(cudaMemcpyAsync(u, s->stage64, n * 8, cudaMemcpyDeviceToHost, s->stream));
-    } else {
-        tmp.resize(n);
-        FR_CK(cudaMemcpyAsync(tmp.data(), s->stage64, n * 8, cudaMemcpyDeviceToHost, s->stream));
-    }
+    FR_CK(cudaMemcpyAsync(u, s->stage64 + so, (size_t)s->inst_nsp[inst] * s->V * 8, cudaMemcpyDeviceToHost, s->stream));
     return FR_OK;
 }
 
-void finish_download(const fr_solver *s, int inst, const std::vector<double> &tmp, double *u) {
-    if (!spread(s, inst)) return;
-    const int V = s->V;
-    std::vector<int64_t> blk(s->grp.size());
-    for (size_t g = 0; g < s->grp.size(); ++g) blk[g] = stage_block(s, inst, (int)g);
-    for (size_t e = 0; e < s->egroup[inst].size(); ++e) {
-        const int g = s->egroup[inst][e];
-        const size_t cnt = (size_t)s->grp[g].nsp * V;
-        std::memcpy(u + s->esp[inst][e] * V, &tmp[blk[g] + s->elocal[inst][e] * cnt], cnt * 8);
-    }
-}
-
-// Whole-batch staging (every instance in one degree group, the usual case):
-// one copy of all instances' FP64 states each way through the FP64 staging
-// buffer, which holds the batch in the ABI's order; the conversions run over
-// runs of instances that are consecutive both there and in their group.
-bool batch_stageable(const fr_solver *s) {
-    for (int i = 0; i < s->n_inst; ++i)
-        if (spread(s, i)) return false;
-    return true;
-}
-
+// Whole-batch transfers: one copy of all instances' FP64 states each way
+// through the FP64 staging buffer, which holds the batch in the ABI's order.
+// Where every instance lies in one degree group the conversions run over runs
+// of instances that are consecutive both there and in their group; in a batch
+// with instances spread over several groups over each group's elements, which
+// find their place in the staging buffer by a table (a host reorder of such
+// instances took 14 ms for 118 MB).
 // Runs of consecutive instances in [i0, i1) that are consecutive both in the
 // staging buffer and in their degree group: fn(group, first element, elements,
 // staging offset in doubles).
 template <typename F>
 fr_status for_instance_runs(const fr_solver *s, int i0, int i1, F &&fn) {
     const int V = s->V;
+    if (s->mapped) {
+        for (size_t g = 0; g < s->grp.size(); ++g) {
+            int64_t ne = 0;
+            for (int i = i0; i < i1; ++i) ne += s->grp[g].ne[i];
+            if (ne > 0) FR_TRY(fn((int)g, s->grp[g].off[i0], ne, (int64_t)0));
+        }
+        return FR_OK;
+    }
     int g_run = -1;
     int64_t e0 = 0, ne = 0, so = 0, off = 0;
     for (int i = 0; i < i0; ++i) off += s->inst_nsp[i] * V;
@@ -1714,7 +1710,7 @@ cudaError_t ensure_xfer(fr_solver *s) {
     return e;
 }
 
-// face data of the instances [i0, i1) (each in one degree group)
+// face data of the instances [i0, i1)
 fr_status enqueue_faces_of(fr_solver *s, int i0, int i1) {
     for (size_t g = 0; g < s->grp.size(); ++g) {
         const Group &G = s->grp[g];
@@ -1756,17 +1752,12 @@ fr_status enqueue_upload_batch(fr_solver *s, const double *u) {
     for (size_t c = 0; c < ch.size(); ++c) {
         FR_CK(cudaStreamWaitEvent(s->stream, s->xev[c], 0));
         FR_TRY(for_instance_runs(s, ch[c].i0, ch[c].i1, [&](int g, int64_t e0, int64_t ne, int64_t so) -> fr_status {
-            Launch cv;
-            cv.kind = frk::K_TO_REAL;
-            cv.g = g;
-            cv.elem0 = e0;
-            cv.n_elem = ne;
-            cv.stage_off = so;
-            cv.grid = grid_for(ne * s->grp[g].nsp * s->V);
-            FR_CK(launch(s, cv));
-            return FR_OK;
+            return convert(s, frk::K_TO_REAL, 0, g, e0, ne, so);
         }));
         FR_TRY(enqueue_faces_of(s, ch[c].i0, ch[c].i1));
+        int64_t faces = 0;
+        for (int i = ch[c].i0; i < ch[c].i1; ++i) faces += s->mcnt[i];
+        FR_CK(mortar_traces(s, s->parity, s->moff[ch[c].i0], faces));
     }
     return FR_OK;
 }
@@ -1779,16 +1770,7 @@ fr_status enqueue_download_batch(fr_solver *s, int src, double *u) {
     const std::vector<XferChunk> ch = xfer_chunks(s);
     for (size_t c = 0; c < ch.size(); ++c) {
         FR_TRY(for_instance_runs(s, ch[c].i0, ch[c].i1, [&](int g, int64_t e0, int64_t ne, int64_t so) -> fr_status {
-            Launch cv;
-            cv.kind = frk::K_TO_F64;
-            cv.g = g;
-            cv.elem0 = e0;
-            cv.n_elem = ne;
-            cv.integral_src = src;
-            cv.stage_off = so;
-            cv.grid = grid_for(ne * s->grp[g].nsp * s->V);
-            FR_CK(launch(s, cv));
-            return FR_OK;
+            return convert(s, frk::K_TO_F64, src, g, e0, ne, so);
         }));
         FR_CK(cudaEventRecord(s->xev[c], s->stream));
         FR_CK(cudaStreamWaitEvent(s->xfer, s->xev[c], 0));
@@ -1807,72 +1789,40 @@ extern "C" fr_status fr_set_state(fr_solver *s, int inst, const double *u) {
     fr_status st = check_inst(s, inst);
     if (st != FR_OK) return st;
     if (!u) { set_error("null state"); return FR_ERR_INVALID_ARG; }
-    std::vector<double> tmp;
-    st = enqueue_upload(s, inst, u, tmp);
+    st = enqueue_upload(s, inst, u);
     if (st != FR_OK) return st;
     FR_CK(cudaStreamSynchronize(s->stream));
     return FR_OK;
 }
 
 static fr_status copy_out(fr_solver *s, int inst, int src, double *u) {
-    std::vector<double> tmp;
-    fr_status st = enqueue_download(s, inst, src, u, tmp);
+    fr_status st = enqueue_download(s, inst, src, u);
     if (st != FR_OK) return st;
     FR_CK(cudaStreamSynchronize(s->stream));
-    finish_download(s, inst, tmp, u);
     return FR_OK;
 }
 
 extern "C" fr_status fr_set_states(fr_solver *s, const double *u) {
     fr::Range nvtx_range("fr_set_states");
     if (!s || !u) { set_error("null argument"); return FR_ERR_INVALID_ARG; }
-    if (batch_stageable(s)) {
-        fr_status st = enqueue_upload_batch(s, u);
-        cudaError_t e = cudaStreamSynchronize(s->stream);   // the host array must outlive the copy
-        // (on an error return the solver stream may not have waited for every
-        // copy already issued on the transfer stream)
-        if (s->xfer) cudaStreamSynchronize(s->xfer);
-        if (st != FR_OK) return st;
-        FR_CK(e);
-        return FR_OK;
-    }
-    std::vector<std::vector<double>> tmp(s->n_inst);
-    size_t off = 0;
-    for (int i = 0; i < s->n_inst; ++i) {
-        fr_status st = enqueue_upload(s, i, u + off, tmp[i]);
-        if (st != FR_OK) {
-            cudaStreamSynchronize(s->stream);   // the host buffers above must outlive the copies
-            return st;
-        }
-        off += (size_t)s->inst_nsp[i] * s->V;
-    }
-    FR_CK(cudaStreamSynchronize(s->stream));
+    fr_status st = enqueue_upload_batch(s, u);
+    cudaError_t e = cudaStreamSynchronize(s->stream);   // the host array must outlive the copy
+    // (on an error return the solver stream may not have waited for every
+    // copy already issued on the transfer stream)
+    if (s->xfer) cudaStreamSynchronize(s->xfer);
+    if (st != FR_OK) return st;
+    FR_CK(e);
     return FR_OK;
 }
 
 extern "C" fr_status fr_get_states(fr_solver *s, double *u) {
     fr::Range nvtx_range("fr_get_states");
     if (!s || !u) { set_error("null argument"); return FR_ERR_INVALID_ARG; }
-    if (batch_stageable(s)) {
-        fr_status st = enqueue_download_batch(s, 0, u);
-        cudaError_t e = cudaStreamSynchronize(s->stream);
-        if (s->xfer) cudaStreamSynchronize(s->xfer);   // as in fr_set_states
-        if (st != FR_OK) return st;
-        FR_CK(e);
-        return FR_OK;
-    }
-    std::vector<std::vector<double>> tmp(s->n_inst);
-    std::vector<size_t> off(s->n_inst + 1, 0);
-    for (int i = 0; i < s->n_inst; ++i) off[i + 1] = off[i] + (size_t)s->inst_nsp[i] * s->V;
-    for (int i = 0; i < s->n_inst; ++i) {
-        fr_status st = enqueue_download(s, i, 0, u + off[i], tmp[i]);
-        if (st != FR_OK) {
-            cudaStreamSynchronize(s->stream);
-            return st;
-        }
-    }
-    FR_CK(cudaStreamSynchronize(s->stream));
-    for (int i = 0; i < s->n_inst; ++i) finish_download(s, i, tmp[i], u + off[i]);
+    fr_status st = enqueue_download_batch(s, 0, u);
+    cudaError_t e = cudaStreamSynchronize(s->stream);
+    if (s->xfer) cudaStreamSynchronize(s->xfer);   // as in fr_set_states
+    if (st != FR_OK) return st;
+    FR_CK(e);
     return FR_OK;
 }
 
@@ -2564,9 +2514,9 @@ extern "C" fr_status fr_tune(fr_solver *s, const char *cache_path, int mode, cha
         }
         u0[V - 1] = s->cfg.p_inf / (s->cfg.gamma - 1.0) + 0.5 * s->cfg.rho_inf * v2;
         for (int i = 0; i < s->n_inst; ++i) {
-            std::vector<double> fs((size_t)s->inst_nsp[i] * V), tmp;
+            std::vector<double> fs((size_t)s->inst_nsp[i] * V);
             for (size_t q = 0; q < fs.size(); ++q) fs[q] = u0[q % V];
-            fr_status su = enqueue_upload(s, i, fs.data(), tmp);
+            fr_status su = enqueue_upload(s, i, fs.data());
             if (su != FR_OK) return su;
             FR_CK(cudaStreamSynchronize(s->stream));
         }

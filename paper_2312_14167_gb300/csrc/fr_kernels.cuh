@@ -166,6 +166,7 @@ struct KArgs {
     double *force_acc;         // [n_inst][3]
     const double *stage64;     // FP64 staging in
     double *stage64_out;       // FP64 staging out
+    const int64_t *EOFF;       // null, or every element's offset in the staging buffer
     double *partials;          // [blocks][2*V + 1]
     double *reduce_out;        // [2*V + 1]
     int64_t n_partials;
@@ -2657,6 +2658,24 @@ __global__ void k_to_real(const KArgs<real> a) {
     // FP32: store the perturbation about the reference state
     auto ref = [&](int64_t i) { return sizeof(real) == 4 ? a.uref64[i % V] : 0.0; };
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+    if (a.EOFF) {
+        // elements in an order of their own: the element's block is contiguous
+        constexpr int PER = G::NSP * V;
+        for (int64_t k0 = t0; k0 < total; k0 += nt * kConvPairs) {
+            double x[kConvPairs];
+#pragma unroll
+            for (int c = 0; c < kConvPairs; ++c) {
+                const int64_t k = k0 + c * nt;
+                if (k < total) x[c] = a.stage64[a.EOFF[a.elem0 + k / PER] + k % PER];
+            }
+#pragma unroll
+            for (int c = 0; c < kConvPairs; ++c) {
+                const int64_t k = k0 + c * nt;
+                if (k < total) a.U[off + k] = (real)(x[c] - ref(k));
+            }
+        }
+        return;
+    }
     if (((total | off) & 1) == 0 && (reinterpret_cast<uintptr_t>(a.stage64) & 15) == 0) {
         const double2 *src = reinterpret_cast<const double2 *>(a.stage64);
         const int64_t np = total / 2;
@@ -2688,6 +2707,21 @@ __global__ void k_to_f64(const KArgs<real> a) {
     const bool shift = sizeof(real) == 4 && !a.integral_src;
     auto ref = [&](int64_t i) { return shift ? a.uref64[i % V] : 0.0; };
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+    if (a.EOFF) {
+        constexpr int PER = G::NSP * V;
+        for (int64_t k0 = t0; k0 < total; k0 += nt * kConvPairs) {
+            real x[kConvPairs];
+#pragma unroll
+            for (int c = 0; c < kConvPairs; ++c)
+                if (k0 + c * nt < total) x[c] = src[off + k0 + c * nt];
+#pragma unroll
+            for (int c = 0; c < kConvPairs; ++c) {
+                const int64_t k = k0 + c * nt;
+                if (k < total) a.stage64_out[a.EOFF[a.elem0 + k / PER] + k % PER] = (double)x[c] + ref(k);
+            }
+        }
+        return;
+    }
     if (((total | off) & 1) == 0 && (reinterpret_cast<uintptr_t>(a.stage64_out) & 15) == 0) {
         double2 *dst = reinterpret_cast<double2 *>(a.stage64_out);
         const int64_t np = total / 2;
