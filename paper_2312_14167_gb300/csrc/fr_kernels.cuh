@@ -132,6 +132,7 @@ template <typename real>
 struct KArgs {
     int64_t n_elem;            // elements (or list entries) in the launch
     int64_t elem0;             // first element of the launch range
+    int pdl;                   // line kernels: may start before the previous launch ends (host-side choice)
     int tile;                  // elements per CTA of the tile kernels, at most Geo::NE (tile_elems)
     const int32_t *elist;      // optional element list (force sampling)
     real *U, *R1, *R2, *RES;
@@ -3279,7 +3280,18 @@ cudaError_t launch_n(int kind, bool visc, const KArgs<real> &in, int grid_hint, 
             else k = k_line3<N>;   // one register level: two CTAs per SM by shared memory
             cudaError_t err = prep_smem(k, L::BYTES);
             if (err != cudaSuccess) return err;
-            k<<<(unsigned)((a.n_elem + L::EPB - 1) / L::EPB), L::TH, L::BYTES, st>>>(b);
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)((a.n_elem + L::EPB - 1) / L::EPB));
+            cfg.blockDim = dim3(L::TH);
+            cfg.dynamicSmemBytes = L::BYTES;
+            cfg.stream = st;
+            cudaLaunchAttribute at = {};
+            at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            at.val.programmaticStreamSerializationAllowed = 1;
+            cfg.attrs = &at;
+            cfg.numAttrs = a.pdl ? 1 : 0;
+            err = cudaLaunchKernelEx(&cfg, k, b);
+            if (err != cudaSuccess) return err;
         }
     } else if (kind == K_STAGE) {
         if (a.n_elem <= 0) return cudaSuccess;

@@ -384,7 +384,7 @@ __device__ __forceinline__ V4 mul4(const float2 c, const float *x) {
 // (xi line) and one column (eta line) of its element.  Everything the warp
 // reads is contiguous in memory, so it is fetched at the start with 16-byte
 // asynchronous copies into the warp's part of shared memory (two groups:
-// state + metric terms, face data) and read from there; the new state and
+// geometry + state, partners' face data) and read from there; the new state and
 // register go back as whole sectors.  Lanes reading rows or columns directly
 // (64-byte steps) took more cycles of the L1 data stage than the shared
 // memory traffic of the whole kernel.
@@ -400,6 +400,14 @@ __device__ __forceinline__ void cp4(void *dst, const void *src) {
 __device__ __forceinline__ void cp8(void *dst, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
                  : "memory");
+}
+// Programmatic launches (2-D): a stage kernel may start while the one before it
+// is still running.  What it fetches before pdl_wait is constant; everything
+// the previous stage wrote, and every store of its own, comes after.  (Hexes
+// measured 5-10 % slower that way and are launched as before.)
+__device__ __forceinline__ void pdl_wait() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 __device__ __forceinline__ void prefetch_l2(const void *src) {
     asm volatile("prefetch.global.L2 [%0];" ::"l"(src));
@@ -467,7 +475,6 @@ k_line2(const __grid_constant__ KArgs<float> a) {
             }
         }
     };
-    copy_points(L::oU, a.U);
     {
         const real *src = a.MET + e0 * (NSP * MS);
         real *dst = reinterpret_cast<real *>(sm + L::oM);
@@ -482,25 +489,25 @@ k_line2(const __grid_constant__ KArgs<float> a) {
             for (int it = lane; it < ne * per; it += 32) cp4(dst + it, src + it);
         }
     }
-    cp_commit();
-    {
 #pragma unroll
-        for (int i = 0; i < (2 * L::NF + 31) / 32; ++i) {
-            const int it = lane + 32 * i;
-            if (it < ne * 2 * NFP) {
-                const int j = it / (2 * NFP), q = it % (2 * NFP);
-                cp16(sm + L::oGEO + L::template fp<8>(j, q / N, q % N), a.FGEO + (e0 * 2 * NFP + it) * 4);
-            }
+    for (int i = 0; i < (2 * L::NF + 31) / 32; ++i) {
+        const int it = lane + 32 * i;
+        if (it < ne * 2 * NFP) {
+            const int j = it / (2 * NFP), q = it % (2 * NFP);
+            cp16(sm + L::oGEO + L::template fp<8>(j, q / N, q % N), a.FGEO + (e0 * 2 * NFP + it) * 4);
         }
-        if (!faces_only) {
+    }
+    pdl_wait();
+    copy_points(L::oU, a.U);
+    cp_commit();
+    if (!faces_only) {
 #pragma unroll
-            for (int i = 0; i < (L::NF + 31) / 32; ++i) {
-                const int it = lane + 32 * i;
-                if (it < ne * NFP) {
-                    const int j = it / NFP, q = it % NFP, sl = L::template fp<4>(j, q / N, q % N);
-                    cp16(sm + L::oUF + sl, a.UFin + (e0 * NFP + it) * V);
-                    cp16(sm + L::oFV + sl, a.FVin + (e0 * NFP + it) * V);
-                }
+        for (int i = 0; i < (L::NF + 31) / 32; ++i) {
+            const int it = lane + 32 * i;
+            if (it < ne * NFP) {
+                const int j = it / NFP, q = it % NFP, sl = L::template fp<4>(j, q / N, q % N);
+                cp16(sm + L::oUF + sl, a.UFin + (e0 * NFP + it) * V);
+                cp16(sm + L::oFV + sl, a.FVin + (e0 * NFP + it) * V);
             }
         }
     }
