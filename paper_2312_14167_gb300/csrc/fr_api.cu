@@ -489,7 +489,7 @@ struct Launch {
     int64_t partial_slot = 0;     // first partial-sum block of the launch
     int64_t n_partials = 0;       // K_REDUCE: partial-sum blocks to reduce
     int grid = 1;
-    bool pdl = false;             // line kernels: programmatic launch after a line kernel
+    bool pdl = false;             // programmatic launch after a stage kernel
     cudaStream_t stream = nullptr;   // null: the solver's
 };
 
@@ -676,6 +676,7 @@ int grid_for(int64_t items) {
 fr_status enqueue_eval(fr_solver *s, int par, int mode, double rk_a, double rk_b, double rk_c, int64_t &cnt,
                        bool follows = false) {
     const int G = (int)s->grp.size();
+    const bool serial = s->capturing && G == 1 && s->n_mortar == 0;
     if (s->visc && !s->fused) {
         std::vector<Launch> ls;
         for (int g = G - 1; g >= 0; --g) {
@@ -684,6 +685,7 @@ fr_status enqueue_eval(fr_solver *s, int par, int mode, double rk_a, double rk_b
             l.g = g;
             l.n_elem = s->grp[g].E;
             l.UFin = s->grp[g].UF[par];
+            l.pdl = serial && follows;
             ls.push_back(l);
         }
         FR_TRY(launch_all(s, ls, cnt));
@@ -706,10 +708,11 @@ fr_status enqueue_eval(fr_solver *s, int par, int mode, double rk_a, double rk_b
         f.rk_a = rk_a;
         f.rk_b = rk_b;
         f.rk_c = rk_c;
-        // 2-D, one group, conforming faces: the launch before is the previous
-        // stage's line kernel (50 steps of 31,722 quads 7.14 -> 7.01 ms, 20 of
-        // 4,096 0.811 -> 0.797; hexes lose 5-10 %)
-        f.pdl = follows && s->capturing && s->fused && s->dim == 2 && G == 1 && s->n_mortar == 0;
+        // One group, conforming faces: the launch before is the previous
+        // stage's kernel or, in the split schedule, this stage's gradient
+        // kernel (50 steps of 31,722 quads 7.14 -> 7.01 ms; the 3-D line
+        // kernel loses 5-10 %)
+        f.pdl = s->fused ? follows && serial && s->dim == 2 : serial && (s->visc || follows);
         fs.push_back(f);
     }
     FR_TRY(launch_all(s, fs, cnt));
@@ -794,7 +797,7 @@ fr_status enqueue_attempt(fr_solver *s, int p0, int64_t *n_launch) {
     FR_TRY(enqueue_faces(s, par, cnt));
     const int modes[3] = {frk::M_BS_2, frk::M_BS_3, frk::M_BS_4};
     for (int st = 0; st < 3; ++st) {
-        FR_TRY(enqueue_eval(s, par, modes[st], 0.0, 0.0, 0.0, cnt));
+        FR_TRY(enqueue_eval(s, par, modes[st], 0.0, 0.0, 0.0, cnt, st > 0));
         par ^= 1;
     }
     for (size_t g = 0; g < s->grp.size(); ++g) {

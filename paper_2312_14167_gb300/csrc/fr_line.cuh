@@ -401,14 +401,6 @@ __device__ __forceinline__ void cp8(void *dst, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
                  : "memory");
 }
-// Programmatic launches (2-D): a stage kernel may start while the one before it
-// is still running.  What it fetches before pdl_wait is constant; everything
-// the previous stage wrote, and every store of its own, comes after.  (Hexes
-// measured 5-10 % slower that way and are launched as before.)
-__device__ __forceinline__ void pdl_wait() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
 __device__ __forceinline__ void prefetch_l2(const void *src) {
     asm volatile("prefetch.global.L2 [%0];" ::"l"(src));
 }
