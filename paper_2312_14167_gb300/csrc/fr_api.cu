@@ -220,6 +220,12 @@ bool fusable_batch(int dim, bool fp64, bool visc, bool adapt, const fr_config &c
     return visc && cfg.viscous_scheme == FR_VISC_BR2 && (n_mortar == 0 || (dim == 2 && !fp64 && !adapt));
 }
 
+// LDG stages of 2-D FP32 batches with conforming faces run the line kernels
+// of the gradient + flux pair (fixed steps)
+bool ldg_line_batch(int dim, bool fp64, bool visc, bool adapt, const fr_config &cfg, int64_t n_mortar) {
+    return visc && cfg.viscous_scheme == FR_VISC_LDG && n_mortar == 0 && dim == 2 && !fp64 && !adapt;
+}
+
 // propagate a failed fr_status
 #define FR_TRY(call)                      \
     do {                                  \
@@ -425,6 +431,7 @@ void fill_args(const fr_solver *s, int g, frk::KArgs<real> &a) {
     a.FLAGS = s->FLAGS;
     a.LFP = (const real *)G.LFP;
     a.FGEO = (const float *)G.FGEO;
+    a.ldg_line = ldg_line_batch(s->dim, s->fp64, s->visc, s->adapt, s->cfg, s->n_mortar) ? 1 : 0;
     a.METL = (const float *)G.METL;
     a.EOFF = s->mapped ? G.EOFF : nullptr;
     a.kq = (real)((s->visc ? s->cfg.mu : 0.0) * s->cfg.gamma / (s->cfg.prandtl > 0 ? s->cfg.prandtl : 1.0));
@@ -470,6 +477,7 @@ void fill_args(const fr_solver *s, int g, frk::KArgs<real> &a) {
     for (int i = 0; i < 2 * frk::kMaxN; ++i) a.rL2[i] = pair(a.rL[i]);
     for (int i = 0; i < frk::kMaxN; ++i) {
         a.rGLm2[i] = pair(-a.rGL[i]);
+        a.rGL2[i] = pair(a.rGL[i]);
         a.rGR2[i] = pair(a.rGR[i]);
     }
 }
@@ -1435,7 +1443,7 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
     const bool fusable = fusable_batch(dim, s->fp64, s->visc, s->adapt, *cfg, P.n_mortar);
     s->fused = fusable && !s->fp64 && !s->adapt;
     for (int g = 0; g < P.G; ++g) s->fused = s->fused && (dim == 2 || s->grp[g].N >= 2);
-    if (fusable) {
+    if (fusable || ldg_line_batch(dim, s->fp64, s->visc, s->adapt, *cfg, P.n_mortar)) {
         // partner lifting coefficients per own flux point (FP64, then cast):
         // lf = sum_m l_m(side) g'_side(m) (1/J) S[k][:] along the partner's line
         for (int g = 0; g < P.G; ++g) {

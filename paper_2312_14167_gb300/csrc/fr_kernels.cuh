@@ -182,8 +182,9 @@ struct KArgs {
     double opW[kMaxN];            // Gauss weights
     // the same in the kernel's precision, read from the constant bank (K_LINE)
     real rD[kMaxN * kMaxN], rDT[kMaxN * kMaxN], rL[2 * kMaxN], rGL[kMaxN], rGR[kMaxN];
-    float2 rD2[kMaxN * kMaxN], rDT2[kMaxN * kMaxN], rL2[2 * kMaxN], rGLm2[kMaxN], rGR2[kMaxN];   // as pairs (c, c); -g_L'
+    float2 rD2[kMaxN * kMaxN], rDT2[kMaxN * kMaxN], rL2[2 * kMaxN], rGLm2[kMaxN], rGL2[kMaxN], rGR2[kMaxN];   // as pairs (c, c); rGLm2: -g_L'
     real kq;                      // gamma mu / Pr
+    int ldg_line;                 // LDG stages run k_ldg2 (host-side choice)
     const float *FGEO;            // packed face geometry of K_LINE [E][face][D][point][4]
     const float *METL;            // K_LINE, 3-D: metric terms, order of metl_word
     // perturbation storage (FP32 kernels): reference state, its FP64
@@ -3276,6 +3277,16 @@ cudaError_t launch_n(int kind, bool visc, const KArgs<real> &in, int grid_hint, 
     // amplifies a change of rounding to 5e-5 of the state within 40 attempts,
     // so its kernels stay as they are, bit for bit)
     const bool line_stage = has_line<D, N, real>() && !a.tc && !ad;
+    if constexpr (D == 2 && has_line<D, N, real>()) {
+        if (a.ldg_line && visc && !a.tc && !ad && !a.force && (kind == K_GRAD || kind == K_FLUX)) {
+            if (a.n_elem <= 0) return cudaSuccess;
+            using L = Line2<N>;
+            auto k = kind == K_GRAD ? k_ldg2<N, false> : k_ldg2<N, true>;
+            const cudaError_t err = prep_smem(k, L::BYTES);
+            if (err != cudaSuccess) return err;
+            return launch_pdl(k, (a.n_elem + L::EPB - 1) / L::EPB, L::TH, L::BYTES, st, a.pdl != 0, a);
+        }
+    }
     if (kind == K_FLUX) {
         if (a.n_elem <= 0) return cudaSuccess;
         const size_t sm = smem_bytes<D, N, real>(K_FLUX, visc, a.tc != 0);

@@ -851,6 +851,514 @@ k_line2(const __grid_constant__ KArgs<float> a) {
 }
 
 // --------------------------------------------------------------------------
+// LDG on 2-D lines.  An LDG face needs both sides' corrected gradients, so a
+// stage stays two kernels, in the layout and with the exchange of K_GRAD and
+// K_FLUX (own viscous normal fluxes in FV, the partner's gathered): FLUX false
+// the corrected gradient and the own viscous normal flux of every flux point,
+// FLUX true the rest of the stage.  The work is split as in k_line2: the
+// corrections of a row or column are its own thread's jumps, so nothing but
+// the lines themselves passes through shared memory.
+// --------------------------------------------------------------------------
+template <int D, typename real>
+__device__ __forceinline__ void ldg_face(const KArgs<real> &a, const LineRef<D, real> &R, const FaceGeo<D, real> &g,
+                                         int64_t gf, const real *uL, real *uR, const real *fvo, const real *fvp,
+                                         real *Fs, real *dd) {
+    constexpr int V = D + 2;
+    const real gm1 = a.gamma - real(1);
+    const bool inner = g.pt >= 0;
+    real uLl[V], uRl[V], ub[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) uLl[v] = uL[v] - R.du[v];
+    if (!inner) {
+        BcIn<D, real> in;
+#pragma unroll
+        for (int v = 0; v < V; ++v) { in.u[v] = uLl[v]; in.du[v] = R.du[v]; }
+#pragma unroll
+        for (int d = 0; d < D; ++d) in.n[d] = g.n[d];
+        const BcPair<D, real> o = bc_call<D, real>(&a, -1 - g.pt, in);
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            uRl[v] = o.ug[v];
+            uR[v] = o.ug[v] + R.du[v];
+            ub[v] = o.ub[v] + R.du[v];
+        }
+    } else {
+#pragma unroll
+        for (int v = 0; v < V; ++v) uRl[v] = uR[v] - R.du[v];
+    }
+    real nn = 0, vnr = 0;
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+        nn += g.n[d] * g.n[d];
+        vnr += R.v[d] * g.n[d];
+    }
+    if (a.flux == 1) {
+        RoeIn<D, real> in;
+#pragma unroll
+        for (int v = 0; v < V; ++v) { in.uL[v] = uLl[v]; in.uR[v] = uRl[v]; in.du[v] = R.du[v]; }
+#pragma unroll
+        for (int d = 0; d < D; ++d) in.n[d] = g.n[d];
+        const RoeOut<D, real> o = roe_call<D, real>(&a, in);
+#pragma unroll
+        for (int v = 0; v < V; ++v) Fs[v] = o.F[v];
+    } else {
+        real ir, vp[D], vel[D], pp, p, FL[V], FR[V];
+        prim_line<D>(uLl, R, gm1, ir, vp, vel, pp, p);
+        const real sL = normal_flux_prim<D>(uLl, vp, vel, pp, p, ir, g.n, vnr, nn, R, a.gamma, FL);
+        prim_line<D>(uRl, R, gm1, ir, vp, vel, pp, p);
+        const real sR = normal_flux_prim<D>(uRl, vp, vel, pp, p, ir, g.n, vnr, nn, R, a.gamma, FR);
+        const real lam = real(0.5) * fmax(sL, sR);
+#pragma unroll
+        for (int v = 0; v < V; ++v) Fs[v] = real(0.5) * (FL[v] + FR[v]) - lam * (uR[v] - uL[v]);
+    }
+    if (inner) {
+        // the side with the smaller point index is the left one
+        const real bs = gf < g.pt ? a.ldg_beta : -a.ldg_beta, pen = a.ldg_tau * sqrt(nn);
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            dd[v] = (real(0.5) - bs) * (uR[v] - uL[v]);
+            Fs[v] += pen * (uL[v] - uR[v]) - ((real(0.5) - bs) * fvo[v] - (real(0.5) + bs) * fvp[v]);
+        }
+    } else {
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            dd[v] = ub[v] - uL[v];
+            Fs[v] -= fvo[v];
+        }
+    }
+}
+
+template <int N, bool FLUX>
+__global__ void __launch_bounds__((Line2<N>::TH), 3)
+k_ldg2(const __grid_constant__ KArgs<float> a) {
+    using L = Line2<N>;
+    using real = float;
+    constexpr int D = 2, V = 4, NSP = L::NSP, NFP = L::NFP, MS = L::MS;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    float4 *sm = reinterpret_cast<float4 *>(smem_raw) + wid * L::SLOTS;
+    const int64_t e0 = a.elem0 + (int64_t)blockIdx.x * L::EPB + wid * L::EPW;
+    const int64_t e_end = a.elem0 + a.n_elem;
+    if (e0 >= e_end) return;                       // whole warps: only warp barriers below
+    const int ne = (int)min((int64_t)L::EPW, e_end - e0);
+    const int mode = a.mode;
+
+    auto copy_points = [&](int o, const real *src) {
+#pragma unroll
+        for (int i = 0; i < (L::NP + 31) / 32; ++i) {
+            const int it = lane + 32 * i;
+            if (it < ne * NSP) {
+                const int j = it / NSP, s = it % NSP;
+                cp16(sm + o + L::pt(j, s / N, s % N), src + (e0 * NSP + it) * V);
+            }
+        }
+    };
+    {
+        const real *src = a.MET + e0 * (NSP * MS);
+        real *dst = reinterpret_cast<real *>(sm + L::oM);
+        constexpr int per = NSP * MS;
+        if (per % 4 == 0) {
+#pragma unroll
+            for (int i = 0; i < (L::EPW * per / 4 + 31) / 32; ++i) {
+                const int it = lane + 32 * i;
+                if (it < ne * (per / 4)) cp16(dst + 4 * it, src + 4 * it);
+            }
+        } else {
+            for (int it = lane; it < ne * per; it += 32) cp4(dst + it, src + it);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < (2 * L::NF + 31) / 32; ++i) {
+        const int it = lane + 32 * i;
+        if (it < ne * 2 * NFP) {
+            const int j = it / (2 * NFP), q = it % (2 * NFP);
+            cp16(sm + L::oGEO + L::template fp<8>(j, q / N, q % N), a.FGEO + (e0 * 2 * NFP + it) * 4);
+        }
+    }
+    pdl_wait();
+    copy_points(L::oU, a.U);
+    cp_commit();
+    {
+#pragma unroll
+        for (int i = 0; i < (L::NF + 31) / 32; ++i) {
+            const int it = lane + 32 * i;
+            if (it < ne * NFP) {
+                const int j = it / NFP, q = it % NFP, sl = L::template fp<4>(j, q / N, q % N);
+                cp16(sm + L::oUF + sl, a.UFin + (e0 * NFP + it) * V);
+                if (FLUX) cp16(sm + L::oFV + sl, a.FV + (e0 * NFP + it) * V);
+            }
+        }
+    }
+    cp_commit();
+
+    // lanes without an element of their own repeat the last one and store nothing
+    const bool live = lane < ne * N;
+    const int j = min(lane / N, ne - 1), l = lane % N;
+    const int64_t e = e0 + j;
+    int ro[N], co[N];                              // slots of this thread's row and column
+#pragma unroll
+    for (int m = 0; m < N; ++m) {
+        ro[m] = L::pt(j, l, m);
+        co[m] = L::pt(j, m, l);
+    }
+    auto ld = [&](int slot, real *o) {
+        const float4 t = sm[slot];
+        o[0] = t.x; o[1] = t.y; o[2] = t.z; o[3] = t.w;
+    };
+    auto st = [&](int slot, const real *o) {
+        if (live) sm[slot] = make_float4(o[0], o[1], o[2], o[3]);
+    };
+    const real *gM = reinterpret_cast<const real *>(sm + L::oM) + (j * N + l) * (N * MS);
+    const real gm1 = a.gamma - real(1), kq = a.kq;
+
+    auto ends = [&](const real (*x)[V], real (*o)[V]) {
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            V4 t = mul4(a.rL2[s * kMaxN], x[0]);
+#pragma unroll
+            for (int m = 1; m < N; ++m) t = fma4(a.rL2[s * kMaxN + m], x[m], t);
+            t.get(o[s]);
+        }
+    };
+    // derivative of a line with the correction of its jumps
+    auto corrected = [&](const real (*x)[V], const real (*dd)[V], real (*d)[V]) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            V4 t = mul4(a.rD2[i * kMaxN], x[0]);
+#pragma unroll
+            for (int m = 1; m < N; ++m) t = fma4(a.rD2[i * kMaxN + m], x[m], t);
+            fma4(a.rGL2[i], dd[0], fma4(a.rGR2[i], dd[1], t)).get(d[i]);
+        }
+    };
+    auto columns = [&](const real (*dd)[V]) {      // the column's corrected derivative into field G
+        real y[N][V], d[N][V];
+#pragma unroll
+        for (int m = 0; m < N; ++m) ld(L::oU + co[m], y[m]);
+        corrected(y, dd, d);
+#pragma unroll
+        for (int m = 0; m < N; ++m) st(L::oG + co[m], d[m]);
+    };
+    // physical gradient at point i of the row from its corrected derivatives
+    auto grad_pt = [&](const real *m, const real *dx, const real *dy, real (*g)[V]) {
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            const real c0 = m[d] * m[4], c1 = m[2 + d] * m[4];
+#pragma unroll
+            for (int v = 0; v < V; ++v) g[d][v] = c0 * dx[v] + c1 * dy[v];
+        }
+    };
+    auto ends_grad = [&](real (*Q)[D][V]) {        // at the column's ends
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            real x[N][V], o[2][V];
+#pragma unroll
+            for (int m = 0; m < N; ++m) ld(L::oG + d * L::NP + co[m], x[m]);
+            ends(x, o);
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+#pragma unroll
+                for (int v = 0; v < V; ++v) Q[s][d][v] = o[s][v];
+        }
+    };
+    auto geo = [&](int f, FaceGeo<D, real> &g) {
+        const float4 A = sm[L::oGEO + L::template fp<8>(j, 2 * f, l)], B = sm[L::oGEO + L::template fp<8>(j, 2 * f + 1, l)];
+        g.n[0] = A.x; g.n[1] = A.y; g.lf[0] = A.z; g.lf[1] = A.w;
+        g.lfp[0] = B.x; g.lfp[1] = B.y; g.pt = __float_as_int(B.z);
+    };
+
+    real u[N][V], ufr[2][V], ufc[2][V];
+    cp_wait<0>();
+    __syncwarp();
+#pragma unroll
+    for (int m = 0; m < N; ++m) ld(L::oU + ro[m], u[m]);
+    ends(u, ufr);
+    {
+        real y[N][V];
+#pragma unroll
+        for (int m = 0; m < N; ++m) ld(L::oU + co[m], y[m]);
+        ends(y, ufc);
+    }
+    auto face_of = [&](int f) { return e * NFP + f * N + l; };
+
+    if constexpr (!FLUX) {
+        // jumps u_c - u_f and the state of the viscous flux (in place of u_f)
+        real ddr[2][V], ddc[2][V];
+        auto jumps = [&](int k, real (*uf)[V], real (*dd)[V]) {
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                FaceGeo<D, real> g;
+                geo(2 * k + s, g);
+                if (g.pt >= 0) {
+                    real uR[V];
+                    ld(L::oUF + L::template fp<4>(j, 2 * k + s, l), uR);
+                    const real c = real(0.5) - (face_of(2 * k + s) < g.pt ? a.ldg_beta : -a.ldg_beta);
+#pragma unroll
+                    for (int v = 0; v < V; ++v) dd[s][v] = c * (uR[v] - uf[s][v]);
+                } else {
+                    BcIn<D, real> in;
+#pragma unroll
+                    for (int v = 0; v < V; ++v) { in.u[v] = uf[s][v]; in.du[v] = 0; }
+#pragma unroll
+                    for (int d = 0; d < D; ++d) in.n[d] = g.n[d];
+                    const BcPair<D, real> o = bc_call<D, real>(&a, -1 - g.pt, in);
+#pragma unroll
+                    for (int v = 0; v < V; ++v) {
+                        dd[s][v] = o.ub[v] - uf[s][v];
+                        uf[s][v] = o.ub[v];
+                    }
+                }
+            }
+        };
+        jumps(0, ufr, ddr);
+        jumps(1, ufc, ddc);
+        columns(ddc);
+        __syncwarp();
+        real Q[2][D][V];
+        {
+            real M[N * MS], dx[N][V];
+            ld_row<N * MS>(gM, M);
+            corrected(u, ddr, dx);
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+#pragma unroll
+                for (int d = 0; d < D; ++d)
+#pragma unroll
+                    for (int v = 0; v < V; ++v) Q[s][d][v] = 0;
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                real dy[V], g[D][V];
+                ld(L::oG + ro[i], dy);
+                grad_pt(M + i * MS, dx[i], dy, g);
+#pragma unroll
+                for (int d = 0; d < D; ++d) {
+                    st(L::oG + d * L::NP + ro[i], g[d]);
+#pragma unroll
+                    for (int s = 0; s < 2; ++s) {
+                        V4 t;
+                        t.set(Q[s][d]);
+                        fma4(a.rL2[s * kMaxN + i], g[d], t).get(Q[s][d]);
+                    }
+                }
+            }
+        }
+        __syncwarp();
+        auto own_flux = [&](int k, const real (*uf)[V]) {
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                FaceGeo<D, real> g;
+                geo(2 * k + s, g);
+                real full[V], vel[D], fv[V];
+                add_ref<V>(a.ref, uf[s], full);
+                const real ir = real(1) / full[0];
+#pragma unroll
+                for (int d = 0; d < D; ++d) vel[d] = full[1 + d] * ir;
+                visc_normal<D>(Q[s], vel, full[V - 1] * ir, a.mu * ir, kq * ir, g.n, fv);
+                if (g.pt < 0 && a.BTAG[-1 - g.pt] == BC_WALL) fv[V - 1] = 0;   // adiabatic wall
+                if (live) st_v<V>(a.FV + face_of(2 * k + s) * V, fv);
+            }
+        };
+        own_flux(0, ufr);
+        ends_grad(Q);
+        own_flux(1, ufc);
+    } else {
+        real Fs[D][2][V], ddr[2][V];
+        LineRef<D, real> R;      // the element's flux reference, its own or the global one
+        {
+            real u0[V];
+            ld(L::oU + L::pt(j, 0, 0), u0);
+            line_ref<D>(a.ref, u0, a.local_ref && !a.DIVREF, a.gamma, R);
+        }
+        // 1) common normal fluxes and jumps at the ends of this thread's row and column
+        auto face_pair = [&](int k, const real (*uf)[V], real (*dd)[V]) {
+            FaceGeo<D, real> g[2];
+            real fvp[2][V] = {};
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                geo(2 * k + s, g[s]);
+                if (g[s].pt >= 0) ld_v<V>(a.FV + (int64_t)g[s].pt * V, fvp[s]);
+            }
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                real uR[V], fvo[V];
+                const int sl = L::template fp<4>(j, 2 * k + s, l);
+                ld(L::oUF + sl, uR);
+                ld(L::oFV + sl, fvo);
+                ldg_face<D>(a, R, g[s], face_of(2 * k + s), uf[s], uR, fvo, fvp[s], Fs[k][s], dd[s]);
+            }
+        };
+        {
+            real ddc[2][V];
+            face_pair(1, ufc, ddc);
+            columns(ddc);
+        }
+        face_pair(0, ufr, ddr);
+        __syncwarp();
+        // the register array of the RK update comes in over the viscous fluxes
+        const bool lsrk = mode == M_LSRK;
+        if (lsrk) copy_points(L::oFV, a.R1);
+        cp_commit();
+
+        // 2) transformed flux at the row's points
+        real f0[N][V], iJ[N];
+        {
+            real M[N * MS], dx[N][V];
+            ld_row<N * MS>(gM, M);
+            corrected(u, ddr, dx);
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const real *m = M + i * MS;
+                iJ[i] = m[4];
+                real dy[V], gr[D][V], F[D][V], t[V];
+                ld(L::oG + ro[i], dy);
+                grad_pt(m, dx[i], dy, gr);
+                line_flux<D>(a, R, u[i], gr, gm1, kq, F);
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    f0[i][v] = m[0] * F[0][v] + m[1] * F[1][v];
+                    t[v] = m[2] * F[0][v] + m[3] * F[1][v];
+                }
+                st(L::oG + ro[i], t);
+            }
+        }
+        __syncwarp();
+
+        // 3) divergence + correction along the column and the row (the flux
+        // polynomial's end values are folded into DT), then the RK update
+        auto line_div = [&](const real (*x)[V], const real (*F2)[V], real (*o)[V]) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                V4 t = fma4(a.rGLm2[i], F2[0], mul4(a.rGR2[i], F2[1]));
+#pragma unroll
+                for (int m = 0; m < N; ++m) t = fma4(a.rDT2[i * kMaxN + m], x[m], t);
+                t.get(o[i]);
+            }
+        };
+        {
+            real y[N][V], o[N][V];
+#pragma unroll
+            for (int m = 0; m < N; ++m) ld(L::oG + co[m], y[m]);
+            line_div(y, Fs[1], o);
+#pragma unroll
+            for (int m = 0; m < N; ++m) st(L::oG + co[m], o[m]);
+        }
+        real dv[N][V];
+        line_div(f0, Fs[0], dv);
+        cp_wait<0>();
+        __syncwarp();
+        const int64_t row = (e * NSP + l * N) * V;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            real x[V];
+            ld(L::oG + ro[i], x);
+#pragma unroll
+            for (int v = 0; v < V; ++v) dv[i][v] += x[v];
+        }
+        if (a.DIVREF) {
+            // the constant reference flux's share of the divergence
+            real dr[N][V];
+            ld_row<N * V>(a.DIVREF + row, &dr[0][0]);
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+#pragma unroll
+                for (int v = 0; v < V; ++v) dv[i][v] += dr[i][v];
+        }
+        if (mode == M_RESIDUAL_J) {
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+#pragma unroll
+                for (int v = 0; v < V; ++v) dv[i][v] = -dv[i][v];
+            if (live) st_row<N * V>(a.RES + row, &dv[0][0]);
+            return;
+        }
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int v = 0; v < V; ++v) dv[i][v] *= -iJ[i];
+        if (mode == M_RESIDUAL) {
+            if (live) st_row<N * V>(a.RES + row, &dv[0][0]);
+            return;
+        }
+        // shared field o back to memory, whole sectors
+        auto write_points = [&](int o, real *dst) {
+#pragma unroll
+            for (int i = 0; i < (L::NP + 31) / 32; ++i) {
+                const int it = lane + 32 * i;
+                if (it < ne * NSP) {
+                    const int jj = it / NSP, s = it % NSP;
+                    reinterpret_cast<float4 *>(dst)[e0 * NSP + it] = sm[o + L::pt(jj, s / N, s % N)];
+                }
+            }
+        };
+        if (mode == M_LSRK_FIRST || mode == M_LSRK) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                real r[V];
+                if (lsrk) {
+                    ld(L::oFV + ro[i], r);
+#pragma unroll
+                    for (int v = 0; v < V; ++v) r[v] = a.rk_a * r[v] + a.dt * dv[i][v];
+                } else {
+#pragma unroll
+                    for (int v = 0; v < V; ++v) r[v] = a.dt * dv[i][v];
+                }
+#pragma unroll
+                for (int v = 0; v < V; ++v) u[i][v] += a.rk_b * r[v];
+                st(L::oFV + ro[i], r);
+                st(L::oU + ro[i], u[i]);
+            }
+            __syncwarp();
+            write_points(L::oFV, a.R1);
+            write_points(L::oU, a.U);
+        } else {
+            if (mode == M_RK4_1) {
+                if (live) {
+                    st_row<N * V>(a.R1 + row, &u[0][0]);
+                    st_row<N * V>(a.R2 + row, &dv[0][0]);
+                }
+#pragma unroll
+                for (int i = 0; i < N; ++i)
+#pragma unroll
+                    for (int v = 0; v < V; ++v) u[i][v] += a.rk_c * dv[i][v];
+            } else {
+                real r1[N][V], r2[N][V];
+                ld_row<N * V>(a.R1 + row, &r1[0][0]);
+                ld_row<N * V>(a.R2 + row, &r2[0][0]);
+                const bool last = mode == M_RK4_4;
+#pragma unroll
+                for (int i = 0; i < N; ++i)
+#pragma unroll
+                    for (int v = 0; v < V; ++v) {
+                        const real acc = last ? r2[i][v] + dv[i][v] : r2[i][v] + real(2) * dv[i][v];
+                        u[i][v] = r1[i][v] + a.rk_c * (last ? acc : dv[i][v]);
+                        r2[i][v] = acc;
+                    }
+                if (live && !last) st_row<N * V>(a.R2 + row, &r2[0][0]);
+            }
+#pragma unroll
+            for (int i = 0; i < N; ++i) st(L::oU + ro[i], u[i]);
+            __syncwarp();
+            write_points(L::oU, a.U);
+        }
+        // 4) the new face states to the partners' inbound slots
+        auto send = [&](int k, const real (*uf)[V]) {
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                FaceGeo<D, real> g;
+                geo(2 * k + s, g);
+                if (live && g.pt >= 0) st_v<V>(a.UFout + (int64_t)g.pt * V, uf[s]);
+            }
+        };
+        ends(u, ufr);
+        send(0, ufr);
+        real y[N][V];
+#pragma unroll
+        for (int m = 0; m < N; ++m) ld(L::oU + co[m], y[m]);
+        ends(y, ufc);
+        send(1, ufc);
+    }
+}
+
+// --------------------------------------------------------------------------
 // 3-D line kernel.  A thread owns line l of each of the three directions of
 // its element.  A state or flux of five variables is one 128-bit vector (rho,
 // rho v) and one word (rho E), in shared memory as in the face buffers.

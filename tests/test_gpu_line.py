@@ -85,3 +85,30 @@ def test_mortar_faces(degrees, flux):
     for _ in range(5):
         u = T.lsrk45_step(disc.residual, u, case.dt)
     assert FC.rel_l2(sol.get_state(0), u) < 1e-6
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+@pytest.mark.parametrize("shape,flux", [((3, 3), "rusanov"), ((11, 3), "roe"), (None, "rusanov"), (None, "roe")])
+def test_ldg_lines(shape, flux, p):
+    """LDG in the line kernels: one tile edge each, and (shape None) small
+    airfoils with walls and far field, the second one off the tile grid."""
+    if shape is None:
+        case, inst = FC.airfoil_case(n_inst=2, p=p), 1
+        case.flux = flux
+    else:
+        case, inst = _case(shape, p, flux=flux), 0
+    case.viscous_scheme = "ldg"
+    sol = FC.lib_solver(case, "fp32")
+    for i in range(len(case.meshes)):
+        disc = FC.oracle_disc(case, i)
+        u = FC.initial_state(case, disc.sol_coords(), i)
+        sol.set_state(i, u)
+    R32, mag = disc.residual(FC.fp32_input(case, u), magnitude=True)
+    err = FC.rel_l2(sol.residual(inst), R32)
+    bound = 16 * EPS32 * np.linalg.norm(mag) / np.linalg.norm(R32)
+    print(f"p={p} {shape} {flux}: {err:.2e} (bound {bound:.2e})")
+    assert err < bound
+    sol.rk_step(3)
+    for _ in range(3):
+        u = T.lsrk45_step(disc.residual, u, case.dt)
+    assert FC.rel_l2(sol.get_state(inst), u) < 1e-6
