@@ -6,9 +6,10 @@ arXiv:2312.14167; the batched-airfoil workload): 32 seeded 2-D O-meshes of
 8k-40k curved quads, p = 3, compressible Navier-Stokes (BR2) at Re_c = 23000,
 M = 0.2, LSRK45, mixed precision (FP32 state/fluxes, FP64 geometry setup and
 FP64 probe/force accumulators), one observer per candidate 2 chords below the
-trailing edge.  A step is one LSRK45 step of every candidate (5 stages x
-(gradient kernel + fused flux/update kernel)) plus the probe and wall-force
-sampling kernels, replayed from a CUDA graph.
+trailing edge.  A step is one LSRK45 step of every candidate (5 stages of one
+fused line kernel, or of a gradient and a flux/update kernel where the tuner
+finds that faster) plus the probe and wall-force sampling kernels, replayed
+from a CUDA graph.
 
 Metric: solution-point RK-stage updates per second (sum over candidates of
 elements x 16 solution points x 5 stages x steps / device time).
@@ -510,10 +511,11 @@ def algorithmic_bytes(E, s, kind, p=None):
         per = (NSP * V * s * (3 + 0.8) + NSP * MS * s + NFP * D * s + NFP * 4 + NFP * V * s
                + 2 * NFP * V * s + NFP * V * s)
     elif kind == "stage":
-        # fused stage: state r+w, RK register (w + r in 4 of 5 stages), metrics,
-        # normals and partner lifting coefficients, partner indices, inbound and
-        # outbound face state and gradient flux part
-        per = (NSP * V * s * (3 + 0.8) + NSP * MS * s + 2 * NFP * D * s + NFP * 4 + 4 * NFP * V * s)
+        # fused stage (line kernels): state r+w, RK register (w + r in 4 of 5
+        # stages), metrics, the face record of 4 dim values (normal, own and
+        # partner lifting coefficients, partner index), inbound and outbound
+        # face state and gradient flux part
+        per = (NSP * V * s * (3 + 0.8) + NSP * MS * s + 4 * NFP * D * s + 4 * NFP * V * s)
     else:
         per = NSP * V * s + NSP * MS * s + NFP * D * s + NFP * 4 + NFP * V * s + NFP * V * s
     return per * E

@@ -379,8 +379,8 @@ fr_status fr_instance_status(fr_solver *solver, int32_t *flags, int *first_bad);
  * (CUDA events) and the fastest is kept.  The
  * result is cached in the JSON file cache_path (NULL: no cache) under a key
  * of the GPU architecture, dimension, degrees, variables, precision,
- * viscous scheme, interface flux, mortar faces and log2 of the solution
- * points.  mode 0: use the cached entry if there is one, else measure and
+ * viscous scheme, interface flux, mortar faces, log2 of the solution points
+ * and whether the batch runs the line kernels.  mode 0: use the cached entry if there is one, else measure and
  * store; 1: always measure and store; 2: use the cached entry if there is
  * one, else keep the current schedule.  Measuring sets every instance to the
  * configuration's free stream and advances it: call fr_tune before

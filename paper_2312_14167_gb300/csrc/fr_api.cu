@@ -1344,8 +1344,35 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
             const Group &G = s->grp[g];
             const int nsp = G.nsp, nfp = G.nfp;
             const int64_t off = G.off[i];
+            // boundary points are numbered element after element: count first,
+            // then fill the tables in parallel
+            std::vector<int64_t> bstart((size_t)m->n_elem + 1, 0);
+            std::vector<char> has_wall((size_t)m->n_elem, 0);
+#pragma omp parallel for schedule(static)
+            for (int64_t e = 0; e < m->n_elem; ++e)
+                for (int f = 0; f < nfp; ++f) {
+                    const size_t lf = (size_t)e * nfp + f;
+                    if (m->partner[lf] < 0 && m->bctag[lf] != kTagMortar) ++bstart[e + 1];
+                    if (m->bctag[lf] == FR_TAG_WALL) has_wall[e] = 1;
+                }
+            for (int64_t e = 0; e < m->n_elem; ++e) {
+                bstart[e + 1] += bstart[e];
+                if (!has_wall[e]) continue;
+                wall[g].push_back((int32_t)(off + e));
+                for (int f = 0; f < nfp; ++f) {
+                    const size_t lf = (size_t)e * nfp + f;
+                    if (m->bctag[lf] != FR_TAG_WALL) continue;
+                    // face quadrature weight: product of the free directions' weights
+                    const int l = f % G.nfpf, n1 = G.N;
+                    const double wf = dim == 2 ? G.ref.w[l] : G.ref.w[l % n1] * G.ref.w[l / n1];
+                    for (int d = 0; d < dim; ++d) s->wall_nsum[(size_t)i * 3 + d] += wf * m->nrm[lf * dim + d];
+                }
+            }
+            int bad = 0;
+#pragma omp parallel for schedule(static) reduction(| : bad)
             for (int64_t e = 0; e < m->n_elem; ++e) {
                 const int64_t ge = off + e;
+                int64_t bp = b + bstart[e];
                 einst[g][ge] = i;
                 for (int sp = 0; sp < nsp; ++sp) {
                     const size_t src = (size_t)e * nsp + sp;
@@ -1353,15 +1380,8 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
                         met[g][((size_t)ge * nsp + sp) * MS + kk] = m->S[src * dim * dim + kk];
                     met[g][((size_t)ge * nsp + sp) * MS + dim * dim] = 1.0 / m->J[src];
                 }
-                bool has_wall = false;
                 for (int f = 0; f < nfp; ++f) {
                     const size_t lf = (size_t)e * nfp + f;
-                    if (m->bctag[lf] == FR_TAG_WALL) {
-                        // face quadrature weight: product of the free directions' weights
-                        const int l = f % G.nfpf, n1 = G.N;
-                        const double wf = dim == 2 ? G.ref.w[l] : G.ref.w[l % n1] * G.ref.w[l / n1];
-                        for (int d = 0; d < dim; ++d) s->wall_nsum[(size_t)i * 3 + d] += wf * m->nrm[lf * dim + d];
-                    }
                     for (int d = 0; d < dim; ++d) nrm[g][((size_t)ge * nfp + f) * dim + d] = m->nrm[lf * dim + d];
                     const int64_t pt = m->partner[lf];
                     const int32_t tag = m->bctag[lf];
@@ -1370,26 +1390,29 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
                     } else if (tag == kTagMortar) {
                         const int64_t b0 = box_start[g][(size_t)ge * nfaces + f / G.nfpf];
                         if (b0 < G.fp_real || b0 + G.nfpf > G.fp_real + G.n_box) {
-                            set_error("face joining two degrees without its mortar record");
-                            return FR_ERR_MESH;
+                            bad = 1;
+                            continue;
                         }
                         part[g][(size_t)ge * nfp + f] = (int32_t)(b0 + f % G.nfpf);
                     } else {
-                        part[g][(size_t)ge * nfp + f] = (int32_t)(-1 - b);
-                        btag[b] = tag;
+                        part[g][(size_t)ge * nfp + f] = (int32_t)(-1 - bp);
+                        btag[bp] = tag;
                         // reference velocity at this point (tanh profile on inflow)
                         double prof = 1.0;
                         if (tag == FR_TAG_INFLOW && cfg->inflow_delta > 0.0)
                             prof = std::tanh(3.0 * (m->x_fp[lf * dim + 1] - cfg->inflow_ywall) / cfg->inflow_delta);
                         // FP32 stores it relative to the reference velocity
                         for (int d = 0; d < dim; ++d)
-                            bvref[(size_t)b * dim + d] = cfg->v_inf[d] * prof - s->vref64[d];
-                        if (tag == FR_TAG_WALL) has_wall = true;
-                        ++b;
+                            bvref[(size_t)bp * dim + d] = cfg->v_inf[d] * prof - s->vref64[d];
+                        ++bp;
                     }
                 }
-                if (has_wall) wall[g].push_back((int32_t)ge);
             }
+            if (bad) {
+                set_error("face joining two degrees without its mortar record");
+                return FR_ERR_MESH;
+            }
+            b += bstart[m->n_elem];
         }
         // slim host copy for probe location
         const fr_mesh *m = meshes[i];
@@ -2419,10 +2442,15 @@ std::string tune_key(const fr_solver *s) {
     int bucket = 0;
     while (((int64_t)1 << (bucket + 1)) <= nsp) ++bucket;
     char buf[256];
-    std::snprintf(buf, sizeof(buf), "sm_%d%d|dim=%d|p=%s|V=%d|%s|%s|%s|mortar=%d|log2sp=%d", prop.major,
+    // batches of the line kernels have entries of their own: a schedule measured
+    // on the tile kernels, or for adaptive steps, is no choice for them
+    const bool line = !s->fp64 && !s->adapt &&
+                      (fusable_batch(s->dim, s->fp64, s->visc, s->adapt, s->cfg, s->n_mortar) ||
+                       ldg_line_batch(s->dim, s->fp64, s->visc, s->adapt, s->cfg, s->n_mortar));
+    std::snprintf(buf, sizeof(buf), "sm_%d%d|dim=%d|p=%s|V=%d|%s|%s|%s|mortar=%d|log2sp=%d%s", prop.major,
                   prop.minor, s->dim, deg.c_str(), s->V, s->fp64 ? "fp64" : "fp32",
                   !s->visc ? "euler" : (s->cfg.viscous_scheme == FR_VISC_LDG ? "ldg" : "br2"),
-                  s->cfg.flux == FR_FLUX_ROE ? "roe" : "rusanov", s->n_mortar > 0 ? 1 : 0, bucket);
+                  s->cfg.flux == FR_FLUX_ROE ? "roe" : "rusanov", s->n_mortar > 0 ? 1 : 0, bucket, line ? "|line" : "");
     return buf;
 }
 
