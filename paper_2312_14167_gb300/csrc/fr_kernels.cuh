@@ -22,7 +22,9 @@
 //  * viscous flows add one kernel per stage that computes the BR2 face
 //    gradient and the own-side viscous normal flux at every flux point;
 //  * FP64 (plain) and FP32 (mixed) are the same templates; geometry arrives
-//    already cast from the FP64 host computation.
+//    already cast from the FP64 host computation;
+//  * FP32 viscous stages with fixed steps run the line kernels of fr_line.cuh
+//    instead (3-D LDG or mortar batches excepted).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -3244,10 +3246,12 @@ cudaError_t prep_smem(K kernel, size_t bytes) {
 // lanes per SM and clock), so a batch of fewer CTAs than SMs leaves most of
 // that pipe idle: 256 quads of p = 2 in 10 full tiles took 26 us per stage, in
 // 128 tiles of 2 elements 10.5 us.  The tile that leaves the busiest SM the
-// fewest warps of solution and flux points is taken, the largest of equals; at
-// full tiles the pipe is evenly loaded from some thousand elements on.  FP32
-// launches are latency-bound at such sizes and gain nothing.
-constexpr int kSMs = 152;
+// fewest warps of solution and flux points is taken, the largest of equals; a
+// CTA counts as three warps more (its barriers and start: without that, 40,000
+// quads of p = 3 were cut into 20,000 CTAs of one warp to even out a last wave,
+// at 1.5 times the time of full tiles).  FP32 launches are latency-bound at
+// such sizes and gain nothing.
+constexpr int kSMs = 152, kCtaWarps = 3;
 template <int D, int N, typename real>
 int tile_elems(int64_t n_elem) {
     using G = Geo<D, N>;
@@ -3256,7 +3260,8 @@ int tile_elems(int64_t n_elem) {
     int64_t least = INT64_MAX;
     for (int t = G::NE; t >= 1; --t) {
         const int64_t ctas = (n_elem + t - 1) / t;
-        const int64_t warps = (ctas + kSMs - 1) / kSMs * ((t * G::NSP + 31) / 32 + (t * G::NFP + 31) / 32);
+        const int64_t warps =
+            (ctas + kSMs - 1) / kSMs * ((t * G::NSP + 31) / 32 + (t * G::NFP + 31) / 32 + kCtaWarps);
         if (warps < least) { least = warps; best = t; }
     }
     return best;

@@ -857,7 +857,9 @@ k_line2(const __grid_constant__ KArgs<float> a) {
 // the corrected gradient and the own viscous normal flux of every flux point,
 // FLUX true the rest of the stage.  The work is split as in k_line2: the
 // corrections of a row or column are its own thread's jumps, so nothing but
-// the lines themselves passes through shared memory.
+// the lines themselves passes through shared memory.  Bound as k_line2 (and by
+// the call of the Roe flux); 20 steps of 26,568 quads of p = 4 with Roe 6.62 ->
+// 4.47 ms against K_GRAD + K_FLUX.
 // --------------------------------------------------------------------------
 template <int D, typename real>
 __device__ __forceinline__ void ldg_face(const KArgs<real> &a, const LineRef<D, real> &R, const FaceGeo<D, real> &g,
@@ -1846,7 +1848,9 @@ k_line3(const __grid_constant__ KArgs<float> a) {
 // sides' own viscous normal fluxes are their gradient part plus the lifting of
 // their jump, the lower side's carried by T; the lower side takes minus the
 // projection of the common flux.  (The gradient + flux pair needs two mortar
-// launches per stage, around the flux kernel.)
+// launches per stage, around the flux kernel.)  Latency-bound, some thousand
+// faces per launch; with it an 8-candidate poll of degrees 3 to 0 runs its
+// stages in line kernels, 1.80 -> 0.87 ms per step.
 // --------------------------------------------------------------------------
 struct MortarLineArgs {
     float *UF[5];                  // face states of the pass, per degree group
