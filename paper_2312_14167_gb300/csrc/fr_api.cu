@@ -498,6 +498,8 @@ struct Launch {
     int64_t n_partials = 0;       // K_REDUCE: partial-sum blocks to reduce
     int grid = 1;
     bool pdl = false;             // programmatic launch after a stage kernel
+    bool tiles = false;           // LDG: K_GRAD / K_FLUX also where the stages run line kernels
+    void *FV = nullptr;           // K_GRAD / K_FLUX: own viscous normal fluxes (null: the group's)
     cudaStream_t stream = nullptr;   // null: the solver's
 };
 
@@ -511,6 +513,8 @@ cudaError_t do_launch(const fr_solver *s, const Launch &L) {
     a.mode = L.mode;
     a.force = L.force;
     a.pdl = L.pdl ? 1 : 0;
+    if (L.tiles) a.ldg_line = 0;
+    if (L.FV) a.FV = (real *)L.FV;
     a.integral_src = L.integral_src;
     a.rk_a = (real)L.rk_a;
     a.rk_b = (real)L.rk_b;
@@ -535,14 +539,17 @@ cudaError_t do_launch(const fr_solver *s, const Launch &L) {
     }
 }
 
+// inbound gradient-flux-part buffer of face parity par (fused stage)
+char *fvbuf(const Group &G, int par) { return par == 0 ? G.FV : G.FV2; }
+
 template <typename real>
-cudaError_t do_mortar(const fr_solver *s, int pass, int par, int64_t m0, int64_t count) {
+cudaError_t do_mortar(const fr_solver *s, int pass, int par, int64_t m0, int64_t count, bool fv_par) {
     frk::MArgs<real> a;
     std::memset(&a, 0, sizeof(a));
     for (size_t g = 0; g < s->grp.size(); ++g) {
         const Group &G = s->grp[g];
         a.UF[g] = (real *)G.UF[par];
-        a.FV[g] = (const real *)G.FV;
+        a.FV[g] = (const real *)(fv_par ? fvbuf(G, par) : G.FV);
         a.NRM[g] = (const real *)G.NRM;
         a.MFLUX[g] = (real *)G.MFLUX;
         a.fp_real[g] = G.fp_real;
@@ -631,16 +638,15 @@ cudaError_t ensure_side(fr_solver *s) {
     return e;
 }
 
-// mortar pass over the faces [m0, m0 + count) on face buffer parity par
-cudaError_t mortar(const fr_solver *s, int pass, int par, int64_t m0, int64_t count) {
+// mortar pass over the faces [m0, m0 + count) on face buffer parity par;
+// fv_par: the viscous normal fluxes are in that parity's gradient-part buffer
+cudaError_t mortar(const fr_solver *s, int pass, int par, int64_t m0, int64_t count, bool fv_par = false) {
     if (count <= 0) return cudaSuccess;
     return timed(s, P_OTHER, [&] {
-        return s->fp64 ? do_mortar<double>(s, pass, par, m0, count) : do_mortar<float>(s, pass, par, m0, count);
+        return s->fp64 ? do_mortar<double>(s, pass, par, m0, count, fv_par)
+                       : do_mortar<float>(s, pass, par, m0, count, fv_par);
     });
 }
-
-// inbound gradient-flux-part buffer of face parity par (fused stage)
-char *fvbuf(const Group &G, int par) { return par == 0 ? G.FV : G.FV2; }
 
 // after the traces of face-buffer parity par have been written: what the next
 // evaluation needs of the mortar faces [m0, m0 + count) (the carried traces;
@@ -896,32 +902,50 @@ fr_status check_inst(fr_solver *s, int inst) {
     return FR_OK;
 }
 
-// residual (or J * residual) of one instance into RES
+// do the stages run the fused line kernels?
+bool line_schedule(const fr_solver *s) { return s->fused && !s->fp64 && !s->adapt && !s->tc; }
+
+// Residual (or J * residual) of one instance into RES.  Where the stages run
+// line kernels it is evaluated by K_GRAD + K_FLUX all the same: in FP32 the
+// energy row of a low-Mach flow is the cancelling divergence of terms of the
+// size H, so that another order of the same sums shows at 1e-5 of the residual
+// (Taylor-Green boxes at M = 0.1, p = 3: 2.6e-5 between the two, 5.77e-5 and
+// 5.80e-5 off the FP64 residual).  A residual then depends on the state alone,
+// not on the schedule.  The face data for it go to the buffers of the other
+// parity, which the next stage writes anew.
 fr_status residual_into_res(fr_solver *s, int inst, int mode) {
     const int G = (int)s->grp.size();
-    if (s->visc && !s->fused) {
+    const bool line = line_schedule(s), fused = s->fused && !line;
+    const int par = line ? s->parity ^ 1 : s->parity;
+    auto each = [&](Launch l) -> fr_status {
         for (int g = 0; g < G; ++g) {
-            Launch l;
-            l.kind = frk::K_GRAD;
+            const Group &gr = s->grp[g];
             l.g = g;
-            l.elem0 = s->grp[g].off[inst];
-            l.n_elem = s->grp[g].ne[inst];
-            l.UFin = s->grp[g].UF[s->parity];
+            l.elem0 = gr.off[inst];
+            l.n_elem = gr.ne[inst];
+            l.UFin = gr.UF[par];
+            l.UFout = gr.UF[par];
+            l.FVin = fvbuf(gr, par);
+            l.FV = line ? fvbuf(gr, par) : nullptr;
+            l.tiles = true;
             FR_CK(launch(s, l));
         }
+        return FR_OK;
+    };
+    Launch in, gr, fl;
+    in.kind = frk::K_INTERP;
+    gr.kind = frk::K_GRAD;
+    fl.kind = fused ? frk::K_STAGE : frk::K_FLUX;
+    fl.mode = mode;
+    if (line) {
+        FR_TRY(each(in));
+        FR_CK(mortar(s, 0, par, s->moff[inst], s->mcnt[inst]));
     }
-    if (!s->fused) FR_CK(mortar(s, 1, s->parity, s->moff[inst], s->mcnt[inst]));
-    for (int g = 0; g < G; ++g) {
-        Launch f;
-        f.kind = s->fused ? frk::K_STAGE : frk::K_FLUX;
-        f.g = g;
-        f.elem0 = s->grp[g].off[inst];
-        f.n_elem = s->grp[g].ne[inst];
-        f.UFin = s->grp[g].UF[s->parity];
-        f.FVin = fvbuf(s->grp[g], s->parity);
-        f.mode = mode;
-        FR_CK(launch(s, f));
-    }
+    if (s->visc && !fused) FR_TRY(each(gr));
+    if (!fused) FR_CK(mortar(s, 1, par, s->moff[inst], s->mcnt[inst], line));
+    FR_TRY(each(fl));
+    // the mortar fluxes of the next stage again
+    if (line) FR_CK(mortar_traces(s, s->parity, s->moff[inst], s->mcnt[inst]));
     return FR_OK;
 }
 

@@ -736,22 +736,10 @@ k_line2(const __grid_constant__ KArgs<float> a) {
 #pragma unroll
                 for (int v = 0; v < V; ++v) dv[i][v] += dr[i][v];
         }
-        if (mode == M_RESIDUAL_J) {
-#pragma unroll
-            for (int i = 0; i < N; ++i)
-#pragma unroll
-                for (int v = 0; v < V; ++v) dv[i][v] = -dv[i][v];
-            if (live) st_row<N * V>(a.RES + row, &dv[0][0]);
-            return;
-        }
 #pragma unroll
         for (int i = 0; i < N; ++i)
 #pragma unroll
             for (int v = 0; v < V; ++v) dv[i][v] *= -iJ[i];
-        if (mode == M_RESIDUAL) {
-            if (live) st_row<N * V>(a.RES + row, &dv[0][0]);
-            return;
-        }
         // shared field o back to memory, whole sectors
         auto write_points = [&](int o, real *dst) {
 #pragma unroll
@@ -1264,22 +1252,10 @@ k_ldg2(const __grid_constant__ KArgs<float> a) {
 #pragma unroll
                 for (int v = 0; v < V; ++v) dv[i][v] += dr[i][v];
         }
-        if (mode == M_RESIDUAL_J) {
-#pragma unroll
-            for (int i = 0; i < N; ++i)
-#pragma unroll
-                for (int v = 0; v < V; ++v) dv[i][v] = -dv[i][v];
-            if (live) st_row<N * V>(a.RES + row, &dv[0][0]);
-            return;
-        }
 #pragma unroll
         for (int i = 0; i < N; ++i)
 #pragma unroll
             for (int v = 0; v < V; ++v) dv[i][v] *= -iJ[i];
-        if (mode == M_RESIDUAL) {
-            if (live) st_row<N * V>(a.RES + row, &dv[0][0]);
-            return;
-        }
         // shared field o back to memory, whole sectors
         auto write_points = [&](int o, real *dst) {
 #pragma unroll
@@ -1782,23 +1758,11 @@ k_line3(const __grid_constant__ KArgs<float> a) {
 #pragma unroll
                 for (int v = 0; v < V; ++v) dv[i][v] += dr[i][v];
         }
-        if (mode == M_RESIDUAL_J) {
-#pragma unroll
-            for (int i = 0; i < N; ++i)
-#pragma unroll
-                for (int v = 0; v < V; ++v) dv[i][v] = -dv[i][v];
-            if (live) st_row<N * V>(a.RES + row, &dv[0][0]);
-            return;
-        }
 #pragma unroll
         for (int i = 0; i < N; ++i) {
             const real iJ = mC[i * LPE].y;
 #pragma unroll
             for (int v = 0; v < V; ++v) dv[i][v] *= -iJ;
-        }
-        if (mode == M_RESIDUAL) {
-            if (live) st_row<N * V>(a.RES + row, &dv[0][0]);
-            return;
         }
         if (mode == M_LSRK_FIRST || mode == M_LSRK) {
 #pragma unroll
