@@ -385,6 +385,8 @@ fr_status fr_instance_status(fr_solver *solver, int32_t *flags, int *first_bad);
  * one, else keep the current schedule.  Measuring sets every instance to the
  * configuration's free stream and advances it: call fr_tune before
  * fr_set_state (it also clears the probe, force and health accumulators).
+ * A cached entry leaves the states as they are and may be taken up at any
+ * time: the face data of the new schedule are derived from them.
  * choice receives "stage=...;regs=...;contract=...;ms=...;source=..." (and, after a
  * measurement, ";candidates=..." with every candidate's ms per step).
  * Synchronises. */

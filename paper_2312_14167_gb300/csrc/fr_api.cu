@@ -2559,7 +2559,12 @@ extern "C" fr_status fr_tune(fr_solver *s, const char *cache_path, int mode, cha
     const std::string key = fr::tune_key(s);
     auto cache = fr::read_cache(cache_path);
     const auto hit = cache.find(key);
+    const bool fused0 = s->fused, tc0 = s->tc;
+    int64_t launches = 0;
     if (mode != 1 && hit != cache.end() && fr::apply_schedule(s, hit->second, "cache")) {
+        // what the face buffers hold and how it is laid out is the schedule's:
+        // derive them again for the states set before this call
+        if (s->fused != fused0 || s->tc != tc0) FR_TRY(enqueue_faces(s, s->parity, launches));
         if (choice && choice_len) std::snprintf(choice, choice_len, "%s", fr::schedule_string(s).c_str());
         return FR_OK;
     }
@@ -2653,6 +2658,7 @@ extern "C" fr_status fr_tune(fr_solver *s, const char *cache_path, int mode, cha
     std::snprintf(v, sizeof(v), "stage=%s;regs=%d;contract=%s;ms=%.6f", best->fused ? "fused" : "split", best->regs,
                   best->tc ? "tc" : "simt", best->ms);
     fr::apply_schedule(s, v, "measured");
+    FR_TRY(enqueue_faces(s, s->parity, launches));   // they are the last candidate's
     std::string all;
     for (const Cand &c : cands) {
         char b[96];
