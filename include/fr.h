@@ -375,8 +375,8 @@ fr_status fr_instance_status(fr_solver *solver, int32_t *flags, int *first_bad);
  * FP32, the contraction of the divergence + correction operators (SIMT
  * sum factorisation, or 3xTF32 tensor-core mma products of every element
  * line: FP32-level accuracy, FP32 accumulation) are measured on the
- * solver's own batch: every candidate runs 2 warm-up and 3 timed RK steps
- * (CUDA events) and the fastest is kept.  The
+ * solver's own batch: every candidate runs 2 warm-up and 3 timed RK steps as
+ * fr_rk_step does (captured steps; CUDA events) and the fastest is kept.  The
  * result is cached in the JSON file cache_path (NULL: no cache) under a key
  * of the GPU architecture, dimension, degrees, variables, precision,
  * viscous scheme, interface flux, mortar faces, log2 of the solution points

@@ -1911,40 +1911,49 @@ extern "C" fr_status fr_residual(fr_solver *s, int inst, double *r) {
     return copy_out(s, inst, 1, r);
 }
 
+namespace fr {
+namespace {
+// One step as fr_rk_step runs it: a replay of the step of the current parity,
+// captured at its first use (plain launches on the NULL stream).
+fr_status run_step(fr_solver *s, int64_t &launched) {
+    const int p0 = s->parity;
+    if (s->stream) {
+        if (!s->graph[p0]) {
+            cudaGraph_t g;
+            FR_CK(ensure_side(s));
+            FR_CK(cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal));
+            int64_t cnt = 0;
+            s->capturing = true;
+            fr_status st = enqueue_step(s, p0, &cnt);
+            s->capturing = false;
+            cudaError_t ce = cudaStreamEndCapture(s->stream, &g);
+            if (st != FR_OK) return st;
+            FR_CK(ce);
+            cudaError_t ie = cudaGraphInstantiate(&s->graph[p0], g, 0);
+            cudaGraphDestroy(g);
+            FR_CK(ie);
+            s->launches_per_step = cnt;
+        }
+        FR_CK(cudaGraphLaunch(s->graph[p0], s->stream));
+        launched += s->launches_per_step;
+    } else {
+        int64_t cnt = 0;
+        FR_TRY(enqueue_step(s, p0, &cnt));
+        launched += cnt;
+    }
+    s->parity = (step_flips(s) % 2) ? p0 ^ 1 : p0;
+    return FR_OK;
+}
+}  // namespace
+}  // namespace fr
+
 extern "C" fr_status fr_rk_step(fr_solver *s, int n_steps) {
     fr::Range nvtx_range("fr_rk_step");
     if (!s || n_steps < 0) { set_error("invalid fr_rk_step arguments"); return FR_ERR_INVALID_ARG; }
-    const int flips = step_flips(s);
     int64_t total = 0;
     if (n_steps > 0) FR_TRY(bs_start_if_needed(s));
     for (int it = 0; it < n_steps; ++it) {
-        const int p0 = s->parity;
-        if (s->stream) {
-            if (!s->graph[p0]) {
-                cudaGraph_t g;
-                FR_CK(ensure_side(s));
-                FR_CK(cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal));
-                int64_t cnt = 0;
-                s->capturing = true;
-                fr_status st = enqueue_step(s, p0, &cnt);
-                s->capturing = false;
-                cudaError_t ce = cudaStreamEndCapture(s->stream, &g);
-                if (st != FR_OK) return st;
-                FR_CK(ce);
-                cudaError_t ie = cudaGraphInstantiate(&s->graph[p0], g, 0);
-                cudaGraphDestroy(g);
-                FR_CK(ie);
-                s->launches_per_step = cnt;
-            }
-            FR_CK(cudaGraphLaunch(s->graph[p0], s->stream));
-            total += s->launches_per_step;
-        } else {
-            int64_t cnt = 0;
-            fr_status st = enqueue_step(s, p0, &cnt);
-            if (st != FR_OK) return st;
-            total += cnt;
-        }
-        s->parity = (flips % 2) ? p0 ^ 1 : p0;
+        FR_TRY(run_step(s, total));
         ++s->steps_since_reset;
         if (s->cfg.check_every > 0 && ++s->steps_since_check >= s->cfg.check_every) {
             s->steps_since_check = 0;
@@ -2579,8 +2588,9 @@ extern "C" fr_status fr_tune(fr_solver *s, const char *cache_path, int mode, cha
     for (int c = 0; c < (s->fp64 ? 1 : 2); ++c)
         for (int f = 0; f < (fusable && !(c == 1 && s->n_mortar > 0) ? 2 : 1); ++f)
             for (int r = 0; r < ((s->fp64 || s->adapt) ? 1 : frk::kRegLevels); ++r) cands.push_back({f == 1, r, c == 1, 0.0});
+    // as fr_rk_step runs them, so that programmatic launches and the parallel
+    // branches of degree groups count (two warm-up steps: both parities' graphs)
     const int warm = 2, timed = 3;
-    const int flips = step_flips(s);
     // every instance starts from the free stream of the configuration
     {
         const int V = s->V;
@@ -2608,27 +2618,11 @@ extern "C" fr_status fr_tune(fr_solver *s, const char *cache_path, int mode, cha
         s->tc = c.tc;
         drop_graphs(s);
         // face data for this schedule, then warm-up and timed steps
-        for (int i = 0; i < s->n_inst && st == FR_OK; ++i) {
-            for (size_t g = 0; g < s->grp.size(); ++g) {
-                const Group &G = s->grp[g];
-                if (G.ne[i] <= 0) continue;
-                Launch in;
-                in.kind = s->fused ? frk::K_INTERP_VISC : frk::K_INTERP;
-                in.g = (int)g;
-                in.elem0 = G.off[i];
-                in.n_elem = G.ne[i];
-                in.UFout = G.UF[s->parity];
-                in.FVout = fvbuf(G, s->parity);
-                if (launch(s, in) != cudaSuccess) st = FR_ERR_CUDA;
-            }
-            if (st == FR_OK && mortar_traces(s, s->parity, s->moff[i], s->mcnt[i]) != cudaSuccess) st = FR_ERR_CUDA;
-        }
+        st = enqueue_faces(s, s->parity, launches);
         if (st == FR_OK) st = bs_start_if_needed(s);
         for (int it = 0; it < warm + timed && st == FR_OK; ++it) {
             if (it == warm && cudaEventRecord(e0, s->stream) != cudaSuccess) st = FR_ERR_CUDA;
-            int64_t cnt = 0;
-            if (st == FR_OK) st = enqueue_step(s, s->parity, &cnt);
-            s->parity = (flips % 2) ? s->parity ^ 1 : s->parity;
+            if (st == FR_OK) st = run_step(s, launches);
         }
         if (st == FR_OK && cudaEventRecord(e1, s->stream) != cudaSuccess) st = FR_ERR_CUDA;
         if (st == FR_OK && cudaEventSynchronize(e1) != cudaSuccess) st = FR_ERR_CUDA;

@@ -81,3 +81,28 @@ def test_measured_schedule_without_a_new_state(name, tmp_path):
     again.rk_step(2)
     a, b = sol.get_states(), again.get_states()
     assert np.linalg.norm(a - b) < 1e-6 * np.linalg.norm(b)
+
+
+def test_measured_time_is_the_steps_time(tmp_path):
+    """The tuner times steps as fr_rk_step runs them: on a batch of four small
+    degree groups (parallel branches of the captured step; one by one they take
+    over twice as long) its time per step is that of the steps that follow,
+    within a half.  The least of five on both sides."""
+    import torch
+    sol = _solver(_box((11, 7)), (0, 1, 2, 3))
+    told = []
+    for _ in range(5):
+        sol.tune(None, mode=1)
+        told.append(float(dict(kv.split("=", 1) for kv in sol.schedule()[0].split(";"))["ms"]))
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    took = []
+    sol.rk_step(3)
+    for _ in range(5):
+        torch.cuda.synchronize()
+        a.record(sol.stream)
+        sol.rk_step(3)
+        b.record(sol.stream)
+        torch.cuda.synchronize()
+        took.append(a.elapsed_time(b) / 3)
+    print(f"told {min(told):.4f} ms, took {min(took):.4f} ms")
+    assert min(told) < 1.5 * min(took)
