@@ -367,11 +367,12 @@ fr_status fr_integral_static(fr_solver *solver, int inst, double *sums, int64_t 
 fr_status fr_instance_status(fr_solver *solver, int32_t *flags, int *first_bad);
 
 /* Autotuner (a service of this library; the paper has no counterpart).  A
- * solver's stage schedule -- for BR2 batches without mortar faces, one
- * fused kernel per RK stage or a gradient kernel plus a flux kernel -- the
+ * solver's stage schedule -- for BR2 batches (with mortar faces: 2-D, FP32,
+ * fixed steps), one fused kernel per RK stage or a gradient kernel plus a flux
+ * kernel -- the
  * register level of its stage kernels (FP32: 0 = the default residency,
- * 1 = one resident CTA fewer per SM and more registers per thread, 2 = one
- * more CTA per SM and fewer registers) and, in
+ * 1 = registers for one resident CTA fewer per SM, 2 = for one more; the fused
+ * FP32 kernel of hexes and the 2-D LDG kernels have one level) and, in
  * FP32, the contraction of the divergence + correction operators (SIMT
  * sum factorisation, or 3xTF32 tensor-core mma products of every element
  * line: FP32-level accuracy, FP32 accumulation) are measured on the

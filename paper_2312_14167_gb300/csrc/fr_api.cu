@@ -2581,13 +2581,17 @@ extern "C" fr_status fr_tune(fr_solver *s, const char *cache_path, int mode, cha
         if (choice && choice_len) std::snprintf(choice, choice_len, "%s", fr::schedule_string(s).c_str());
         return FR_OK;
     }
-    // candidates: stage schedule x register level
+    // candidates: stage schedule x register level (the 3-D line kernel and the
+    // 2-D LDG ones have one level: more would be the same kernels again)
     struct Cand { bool fused; int regs; bool tc; double ms; };
     std::vector<Cand> cands;
     const bool fusable = fusable_batch(s->dim, s->fp64, s->visc, s->adapt, s->cfg, s->n_mortar);
+    const bool ldg_line = ldg_line_batch(s->dim, s->fp64, s->visc, s->adapt, s->cfg, s->n_mortar);
     for (int c = 0; c < (s->fp64 ? 1 : 2); ++c)
-        for (int f = 0; f < (fusable && !(c == 1 && s->n_mortar > 0) ? 2 : 1); ++f)
-            for (int r = 0; r < ((s->fp64 || s->adapt) ? 1 : frk::kRegLevels); ++r) cands.push_back({f == 1, r, c == 1, 0.0});
+        for (int f = 0; f < (fusable && !(c == 1 && s->n_mortar > 0) ? 2 : 1); ++f) {
+            const bool one_level = s->fp64 || s->adapt || (c == 0 && (ldg_line || (f == 1 && s->dim == 3)));
+            for (int r = 0; r < (one_level ? 1 : frk::kRegLevels); ++r) cands.push_back({f == 1, r, c == 1, 0.0});
+        }
     // as fr_rk_step runs them, so that programmatic launches and the parallel
     // branches of degree groups count (two warm-up steps: both parities' graphs)
     const int warm = 2, timed = 3;

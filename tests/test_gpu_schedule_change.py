@@ -106,3 +106,15 @@ def test_measured_time_is_the_steps_time(tmp_path):
         took.append(a.elapsed_time(b) / 3)
     print(f"told {min(told):.4f} ms, took {min(took):.4f} ms")
     assert min(told) < 1.5 * min(took)
+
+
+@pytest.mark.parametrize("scheme", ["br2", "ldg"])
+def test_no_kernel_is_measured_twice(scheme):
+    """The fused kernel of hexes and the 2-D LDG kernels have one register level."""
+    case = _box((3, 4, 3) if scheme == "br2" else (7, 5))
+    case.viscous_scheme = scheme
+    choice = _solver(case).tune(None, mode=1)
+    told = [c.split("=")[0] for c in choice.split("candidates=")[1].split(",")]
+    tc = [f"{s}/{r}/tc" for s in (("split", "fused") if scheme == "br2" else ("split",)) for r in (0, 1, 2)]
+    assert told == (["split/0/simt", "split/1/simt", "split/2/simt", "fused/0/simt"] if scheme == "br2"
+                    else ["split/0/simt"]) + tc
