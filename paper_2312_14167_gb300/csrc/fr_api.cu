@@ -226,6 +226,12 @@ bool ldg_line_batch(int dim, bool fp64, bool visc, bool adapt, const fr_config &
     return visc && cfg.viscous_scheme == FR_VISC_LDG && n_mortar == 0 && dim == 2 && !fp64 && !adapt;
 }
 
+// may the stages of degree p of this batch run line kernels (FP32, fixed steps)?
+bool line_batch(int dim, bool fp64, bool visc, bool adapt, const fr_config &cfg, int64_t n_mortar, int p) {
+    return !fp64 && !adapt && (dim == 2 || p >= 1) &&
+           (fusable_batch(dim, fp64, visc, adapt, cfg, n_mortar) || ldg_line_batch(dim, fp64, visc, adapt, cfg, n_mortar));
+}
+
 // propagate a failed fr_status
 #define FR_TRY(call)                      \
     do {                                  \
@@ -328,7 +334,8 @@ struct Layout {
     size_t ERRE, ADAPT, ACC, ARANGE, total;
 };
 
-Layout make_layout(const Plan &P, int n_inst, bool fp64, bool visc, bool adapt) {
+Layout make_layout(const Plan &P, int n_inst, const fr_config &cfg) {
+    const bool fp64 = cfg.precision == FR_FP64, visc = cfg.viscous != 0, adapt = cfg.rk == FR_BS32;
     const size_t rs = fp64 ? 8 : 4;
     const int dim = P.dim, V = dim + 2, MS = dim * dim + 1;
     Layout L{};
@@ -357,9 +364,10 @@ Layout make_layout(const Plan &P, int n_inst, bool fp64, bool visc, bool adapt) 
         G.FV2 = take(visc ? fc : 16);
         G.LFP = take(visc ? (size_t)E * nfp * dim * rs : 16);
         G.R3 = take(adapt ? st : 16);
-        G.FGEO = take(visc && !fp64 ? (size_t)E * nfp * frk::face_geo(dim) * 4 : 16);
+        const bool line = line_batch(dim, fp64, visc, adapt, cfg, P.n_mortar, P.degree[g]);
+        G.FGEO = take(line ? (size_t)E * nfp * frk::face_geo(dim) * 4 : 16);
         G.EOFF = take(P.spread ? (size_t)E * 8 : 16);
-        G.METL = take(visc && !fp64 && dim == 3 ? (size_t)E * nsp * MS * 4 : 16);
+        G.METL = take(line && dim == 3 ? (size_t)E * nsp * MS * 4 : 16);
     }
     L.BTAG = take((size_t)P.nb * 4);
     L.BVREF = take((size_t)P.nb * dim * rs);
@@ -1143,7 +1151,7 @@ extern "C" size_t fr_workspace_bytes(fr_mesh *const *meshes, int n_inst, const f
     if (check_batch(meshes, n_inst, cfg) != FR_OK) return 0;
     const Plan P = make_plan(meshes, n_inst);
     if (P.G > frk::kMaxGroups) return 0;
-    return make_layout(P, n_inst, cfg->precision == FR_FP64, cfg->viscous != 0, cfg->rk == FR_BS32).total;
+    return make_layout(P, n_inst, *cfg).total;
 }
 
 namespace {
@@ -1203,7 +1211,7 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
             return FR_ERR_UNSUPPORTED;
         }
     }
-    const Layout L = make_layout(P, n_inst, s->fp64, s->visc, s->adapt);
+    const Layout L = make_layout(P, n_inst, *cfg);
     if (ws_bytes < L.total) {
         set_error("workspace too small: need " + std::to_string(L.total) + " bytes");
         return FR_ERR_WORKSPACE;
@@ -1488,8 +1496,9 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
     // on 57,120 of p = 4); elsewhere and for adaptive steps the pair is, and
     // fr_tune measures both
     const bool fusable = fusable_batch(dim, s->fp64, s->visc, s->adapt, *cfg, P.n_mortar);
-    s->fused = fusable && !s->fp64 && !s->adapt;
-    for (int g = 0; g < P.G; ++g) s->fused = s->fused && (dim == 2 || s->grp[g].N >= 2);
+    s->fused = fusable;
+    for (int g = 0; g < P.G; ++g)
+        s->fused = s->fused && line_batch(dim, s->fp64, s->visc, s->adapt, *cfg, P.n_mortar, s->grp[g].p);
     if (fusable || ldg_line_batch(dim, s->fp64, s->visc, s->adapt, *cfg, P.n_mortar)) {
         // partner lifting coefficients per own flux point (FP64, then cast):
         // lf = sum_m l_m(side) g'_side(m) (1/J) S[k][:] along the partner's line
@@ -1516,7 +1525,7 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
                 for (int jd = 0; jd < dim; ++jd) lfp[q * dim + jd] = lf[(size_t)pt * dim + jd];
             }
             FR_CK(up_real(G.LFP, lfp, lfp.size()));
-            if (!s->fp64) {
+            if (line_batch(dim, s->fp64, s->visc, s->adapt, *cfg, P.n_mortar, G.p)) {
                 // the line kernel's face record: normal, own and partner lifting
                 // coefficients times eta, partner index
                 const double eta = cfg->br2_eta > 0 ? cfg->br2_eta : 2.0 * dim;
