@@ -465,28 +465,22 @@ void fill_args(const fr_solver *s, int g, frk::KArgs<real> &a) {
         a.opGL[i] = r.dgL[i];
         a.opGR[i] = r.dgR[i];
         a.opW[i] = r.w[i];
-        a.rL[i] = (real)r.lend[0][i];
-        a.rL[frk::kMaxN + i] = (real)r.lend[1][i];
-        a.rGL[i] = (real)r.dgL[i];
-        a.rGR[i] = (real)r.dgR[i];
-        for (int mm = 0; mm < G.N; ++mm) {
-            a.rD[i * frk::kMaxN + mm] = (real)r.D1[i][mm];
-            a.rDT[i * frk::kMaxN + mm] =
-                (real)(r.D1[i][mm] - r.dgR[i] * r.lend[1][mm] - r.dgL[i] * r.lend[0][mm]);
-        }
         for (int mm = 0; mm < G.N; ++mm)
             a.opDT[i * frk::kMaxN + mm] = r.D1[i][mm] - r.dgR[i] * r.lend[1][mm] - r.dgL[i] * r.lend[0][mm];
     }
-    auto pair = [](real c) { return make_float2((float)c, (float)c); };
+    // the line kernels' (FP32), as pairs (c, c) but for two
+    auto pair = [](double c) { return make_float2((float)c, (float)c); };
     for (int i = 0; i < frk::kMaxN * frk::kMaxN; ++i) {
-        a.rD2[i] = pair(a.rD[i]);
-        a.rDT2[i] = pair(a.rDT[i]);
+        a.rD2[i] = pair(a.opD1[i]);
+        a.rDT2[i] = pair(a.opDT[i]);
     }
-    for (int i = 0; i < 2 * frk::kMaxN; ++i) a.rL2[i] = pair(a.rL[i]);
+    for (int i = 0; i < 2 * frk::kMaxN; ++i) a.rL2[i] = pair(a.opL[i]);
     for (int i = 0; i < frk::kMaxN; ++i) {
-        a.rGLm2[i] = pair(-a.rGL[i]);
-        a.rGL2[i] = pair(a.rGL[i]);
-        a.rGR2[i] = pair(a.rGR[i]);
+        a.rGL[i] = (float)a.opGL[i];
+        a.rGR[i] = (float)a.opGR[i];
+        a.rGLm2[i] = pair(-a.opGL[i]);
+        a.rGL2[i] = pair(a.opGL[i]);
+        a.rGR2[i] = pair(a.opGR[i]);
     }
 }
 

@@ -182,8 +182,8 @@ struct KArgs {
     // in: DT[i][m] = D1[i][m] - g_R'(xi_i) l_m(+1) - g_L'(xi_i) l_m(-1)
     double opDT[kMaxN * kMaxN];
     double opW[kMaxN];            // Gauss weights
-    // the same in the kernel's precision, read from the constant bank (K_LINE)
-    real rD[kMaxN * kMaxN], rDT[kMaxN * kMaxN], rL[2 * kMaxN], rGL[kMaxN], rGR[kMaxN];
+    // the same in FP32, read from the constant bank (K_LINE)
+    float rGL[kMaxN], rGR[kMaxN];
     float2 rD2[kMaxN * kMaxN], rDT2[kMaxN * kMaxN], rL2[2 * kMaxN], rGLm2[kMaxN], rGL2[kMaxN], rGR2[kMaxN];   // as pairs (c, c); rGLm2: -g_L'
     real kq;                      // gamma mu / Pr
     int ldg_line;                 // LDG stages run k_ldg2 (host-side choice)
