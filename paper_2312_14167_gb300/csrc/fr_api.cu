@@ -1482,13 +1482,13 @@ extern "C" fr_status fr_solver_create(fr_solver **out, fr_mesh *const *meshes, i
         }
         FR_CK(cudaMemsetAsync(G.MFLUX, 0, (size_t)G.n_box * s->V * s->rsz, cs));
     }
-    // BR2 stages may run as one fused kernel when every face is conforming.
-    // That is the default where it is a line kernel (FP32, p >= 1: measured
-    // faster than the gradient + flux pair at every size, ms per step 2.50
-    // against 4.89 on 32 airfoil-sized O-meshes of p = 3, 0.142 against 0.236
-    // on 31,722 quads, 3.3 against 5.9 on 48^3 hexes of p = 3, 4.7 against 6.8
-    // on 57,120 of p = 4); elsewhere and for adaptive steps the pair is, and
-    // fr_tune measures both
+    // BR2 stages may run as one fused kernel (fusable_batch).  That is the
+    // default where it is a line kernel (FP32, fixed steps, 3-D p >= 1:
+    // measured faster than the gradient + flux pair at every size, ms per step
+    // 2.50 against 4.89 on 32 airfoil-sized O-meshes of p = 3, 0.142 against
+    // 0.236 on 31,722 quads, 3.3 against 5.9 on 48^3 hexes of p = 3, 4.7
+    // against 6.8 on 57,120 of p = 4); elsewhere the pair is, and fr_tune
+    // measures both
     const bool fusable = fusable_batch(dim, s->fp64, s->visc, s->adapt, *cfg, P.n_mortar);
     s->fused = fusable;
     for (int g = 0; g < P.G; ++g)

@@ -24,7 +24,7 @@
 //  * FP64 (plain) and FP32 (mixed) are the same templates; geometry arrives
 //    already cast from the FP64 host computation;
 //  * FP32 viscous stages with fixed steps run the line kernels of fr_line.cuh
-//    instead (3-D LDG or mortar batches excepted).
+//    instead (3-D LDG or mortar batches excepted); residuals do not.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -3249,8 +3249,8 @@ cudaError_t prep_smem(K kernel, size_t bytes) {
 // fewest warps of solution and flux points is taken, the largest of equals; a
 // CTA counts as three warps more (its barriers and start: without that, 40,000
 // quads of p = 3 were cut into 20,000 CTAs of one warp to even out a last wave,
-// at 1.5 times the time of full tiles).  FP32 launches are latency-bound at
-// such sizes and gain nothing.
+// at 1.5 times the time of full tiles).  FP32 keeps full tiles: its small
+// batches run the line kernels, the remaining tile kernels were not measured.
 constexpr int kSMs = 152, kCtaWarps = 3;
 template <int D, int N, typename real>
 int tile_elems(int64_t n_elem) {
@@ -3278,9 +3278,11 @@ cudaError_t launch_n(int kind, bool visc, const KArgs<real> &in, int grid_hint, 
     const bool l2 = has_level1<N, real>() && a.regs_level == 2;
     constexpr int R1 = has_level1<N, real>() ? 1 : 0, R2 = has_level1<N, real>() ? 2 : 0;
     // FP32 fused stages run the line kernels; the tensor-core option and
-    // adaptive steps keep K_STAGE (an adaptive run on the stability limit
+    // adaptive steps keep K_STAGE.  (An adaptive run on the stability limit
     // amplifies a change of rounding to 5e-5 of the state within 40 attempts,
-    // so its kernels stay as they are, bit for bit)
+    // so FP32 adaptive steps keep the arithmetic of the tile kernels bit for
+    // bit; whether theirs or the line kernels' is nearer to the FP64 run has
+    // not been measured.)
     const bool line_stage = has_line<D, N, real>() && !a.tc && !ad;
     if constexpr (D == 2 && has_line<D, N, real>()) {
         if (a.ldg_line && visc && !a.tc && !ad && !a.force && (kind == K_GRAD || kind == K_FLUX)) {
