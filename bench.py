@@ -154,6 +154,13 @@ NCU_TRAFFIC = {
     "718c2aecf7009444c359541293d3c384c3fcf704339a068bec575a1ab20458a6":
         {"flux_bytes_per_elem": (316.209920e6 + 148.992000e6) / 243854,
          "grad_bytes_per_elem": (249.94e6 + 43.18e6) / 243854},
+    # the same of the split stage, and one launch of the fused line kernel k_line2<4>: the mean
+    # over a step of four stages that read the RK register and one that does not
+    # (profiles/traffic_airfoil8_line_stage.md)
+    "a9ca4b7a25e435a62ea7c4005282606059f22de3ad1057f1f1e5f3f991705484":
+        {"flux_bytes_per_elem": (312.489472e6 + 149.107712e6) / 243854,
+         "grad_bytes_per_elem": (249.933696e6 + 41.985664e6) / 243854,
+         "stage_bytes_per_elem": (0.8 * (452.892845e6 + 205.181440e6) + 0.2 * (390.452480e6 + 202.977536e6)) / 243854},
 }
 
 
@@ -172,6 +179,21 @@ def stage_traffic(schedule, n_elem):
     return (fl + gr) * n_elem if fl and gr else None
 
 
+def line_stage_traffic(schedule, n_elem):
+    """The same of one stage of the fused line kernel."""
+    rec = NCU_TRAFFIC.get(kernel_source_hash())
+    if not rec or W.name != rec.get("workload", "airfoil") or not line_schedule(schedule):
+        return None
+    per_elem = rec.get("stage_bytes_per_elem")
+    return per_elem * n_elem if per_elem else None
+
+
+def line_schedule(schedule):
+    """Does the mixed path run the fused line kernels in this schedule?"""
+    opts = dict(kv.split("=", 1) for kv in schedule.split(";") if "=" in kv)
+    return opts.get("stage") == "fused" and opts.get("contract") == "simt"
+
+
 # FP64 floating-point operations per solution-point stage update of the plain
 # FP64 path (DFMA counted twice, DADD and DMUL once), from an ncu capture of
 # its stage kernels on the 8-candidate airfoil case, valid only for the
@@ -181,6 +203,7 @@ NCU_FP64_FLOPS = {
     # (33,800 quads x 16 points), split schedule; profiles/fp64_stage_airfoil8_flops.md
     "9ce1259f965df7a6229c93f4b0d7905bb8e40b0ec59992f643dadead8b30bb73": (1.9361e8 + 3.6875e8) / (33800 * 16),
     "718c2aecf7009444c359541293d3c384c3fcf704339a068bec575a1ab20458a6": (1.93613e8 + 3.68746e8) / (33800 * 16),
+    "a9ca4b7a25e435a62ea7c4005282606059f22de3ad1057f1f1e5f3f991705484": (1.7792944e8 + 3.1953272e8) / (33800 * 16),
 }
 
 
@@ -715,12 +738,13 @@ def run_gpu(args):
     peak = float(peaks.get("hbm_gbs", 6800.0))
     traffic = None
     rec = NCU_TRAFFIC.get(kernel_source_hash())
-    if rec and W.name == rec.get("workload", "airfoil"):
+    if rec and W.name == rec.get("workload", "airfoil") and (dom_model != "stage" or line_schedule(schedule)):
         per_elem = rec.get(f"{dom_model}_bytes_per_elem")
         traffic = per_elem * E if per_elem else None
     groups = [q for q in range(0, 5) if by_p[q]]
     kbase = "k_stage" if dom_model == "stage" else f"k_{dom}"
-    kname = (f"{kbase}<{W.dim},{W.p + 1},float>" if len(groups) == 1 else
+    kname = (f"k_line{W.dim}<{W.p + 1}>" if dom_model == "stage" and line_schedule(schedule) and len(groups) == 1 else
+             f"{kbase}<{W.dim},{W.p + 1},float>" if len(groups) == 1 else
              f"{kbase}<{W.dim},N,float> over the degree groups N = {[q + 1 for q in groups]}, "
              "one launch each per stage")
     # the whole stage at the method's minimum bytes per update: the bench's
@@ -733,13 +757,15 @@ def run_gpu(args):
     achieved_stage = value / world * b_upd / 1e9
     # measured bytes of one stage over the poll (uniform degree only: the
     # capture is of one degree's kernels)
-    traffic_stage = stage_traffic(schedule, E) if len([q for q in range(0, 5) if by_p[q]]) == 1 else None
+    traffic_stage = None
+    if len([q for q in range(0, 5) if by_p[q]]) == 1:
+        traffic_stage = line_stage_traffic(schedule, E) or stage_traffic(schedule, E)
     roof = {"bound": "hbm", "kernel": "the whole RK stage (every kernel of the step)",
             "achieved": achieved_stage, "peak": peak, "unit": "GB/s", "frac": achieved_stage / peak,
             "traffic": traffic_stage,
             "traffic_bytes_per_update": traffic_stage / NSPT if traffic_stage else None,
-            "traffic_how": ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one split stage "
-                            "(gradient + flux kernel) on 8 of the candidates, scaled to one stage of "
+            "traffic_how": ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one stage (fused line "
+                            "kernel, or gradient + flux kernel) on 8 of the candidates, scaled to one stage of "
                             "the poll by the element count; null when the kernel source, workload or "
                             "schedule differs from the capture's"),
             "bytes_per_update": b_upd, "design_bytes_per_update": design_b,

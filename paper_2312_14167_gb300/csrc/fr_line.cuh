@@ -15,10 +15,11 @@
 // kernels 306 us (1,500 instructions per point, issue slots and phase barriers
 // the bound); one thread per line 193 us (777 instructions; the L1 data stage,
 // 36 % of its cycles on 64-byte-step row accesses); rows and face data fetched
-// by asynchronous copies 164 us; packed FP32 pairs in the contractions 145 us
-// (97 M warp instructions, 53 % of the issue slots, 4.9 TB/s of DRAM traffic =
-// 0.72 of a copy).  What is left: 12 warps per SM (shared memory), each stalled
-// 3.5 cycles per instruction on shared-memory and instruction latency.
+// by asynchronous copies 164 us; packed FP32 pairs in the contractions 144 us
+// (95.5 M warp instructions, 52 % of the issue slots).  243,854 quads of eight
+// airfoils: 142 us and 658 MB of DRAM traffic per stage, 4.65 TB/s = 0.68 of a
+// copy.  What is left: 12 warps per SM (shared memory), each stalled 4.2 cycles
+// per instruction, on shared-memory, global and instruction latency most.
 #pragma once
 
 namespace frk {
@@ -437,7 +438,8 @@ struct Line2 {
 
 template <int N, int RL>
 struct Line2Blocks {
-    // CTAs per SM asked of the register allocator (shared memory holds 3 of p = 3, 4)
+    // CTAs per SM asked of the register allocator (shared memory holds 3 of
+    // p = 3, 4: there level 2 has fewer registers and no CTA more)
     static constexpr int value = RL == 1 ? 2 : RL == 2 ? 4 : 3;
 };
 
@@ -1354,8 +1356,8 @@ k_ldg2(const __grid_constant__ KArgs<float> a) {
 // register level -> this kernel: 48^3 hexes of p = 3 5.32 -> 3.12, 57,120 of
 // p = 4 6.62 -> 4.59.  On the way (p = 3): unrolled, one plane per variable
 // 4.56; loops rolled 3.90; vectors 3.43; staged inputs 3.29; prefetches 3.12.
-// Bound by latency at 8 warps per SM: 44 % of the issue slots, 55 % of the L1
-// data stage, 35 % of DRAM at p = 3.
+// Bound by latency at 8 warps per SM: 45 % of the issue slots, 57 % of the L1
+// data stage, 37 % of DRAM at p = 3.
 // --------------------------------------------------------------------------
 template <int N>
 struct Line3 {
